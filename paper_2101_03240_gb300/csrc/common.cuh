@@ -36,6 +36,7 @@ enum ScratchSlot {
     SC_LITB,      // batched paper-literal invasion: every image's buckets, lists, bit-planes
     SC_LITJ,      // batched paper-literal invasion: job table, statistics, outputs
     SC_BSORT,     // batched invasion: sort job table, presence pool
+    SC_FLOOD,     // invasion by value phases: counters, job table
     SC_NSLOTS
 };
 

@@ -34,6 +34,7 @@
 #include <climits>
 
 #include "common.cuh"
+#include "flood.cuh"
 
 namespace {
 
@@ -42,6 +43,8 @@ constexpr int kNT = 768;         // threads of the persistent CTA (measured: 384
 constexpr int kChunk = 4096;     // voxels per rank-sort chunk (minimum)
 constexpr int kSmemL1Max = 12288;   // level-1 words of one image of a batched call (shared memory)
 constexpr int kNOut = kInvStats;   // int64 outputs of the invasion kernel
+constexpr int64_t kFloodGridVox = 1 << 21;   // images from this size on run by phases on the whole GPU
+constexpr int kFloodCluster = 16;            // CTAs of one image otherwise
 static_assert(64 + kNOut * sizeof(long long) <= kSmallBytes, "output slot too small");
 
 typedef unsigned long long u64;
@@ -2017,6 +2020,87 @@ bool l1_fits_smem(const Inv &a)
     return invade_dyn_smem(a, true) + stat <= (size_t)optin;
 }
 
+// One image by value phases (flood.cu): on the whole GPU when the context has
+// it to itself and the image is large enough to fill it, else on one
+// thread-block cluster.  kFloodGiveUp: the run outgrew its tables and the
+// one-CTA loop has to take the image from the start (a resumed run cannot:
+// its sequence image is partly written by then, so it is copied back first).
+// The tables share the scratch slots of that loop and of the EDT passes.
+int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps, int32_t *seq,
+              int32_t *step_r2, int32_t *step_centre, int64_t cap, int maxd, int npore, const uint8_t *mask, int resume,
+              int64_t k0, int64_t *h_out)
+{
+    cudaStream_t s = ctx->stream;
+    const int64_t N = nvox(d);
+    const JobSizes o = job_sizes(d, npore);
+    const FloodSizes z = ibip_flood_sizes(d, npore, maxd);
+    FloodMem m;
+    m.state = ibip_scratch(ctx, SC_D1, z.state);
+    m.claim = ibip_scratch(ctx, SC_RANK, std::max(o.rank, z.claim));
+    char *a = (char *)ibip_scratch(ctx, SC_OKEY, std::max(o.okey, z.log + z.tables2));
+    char *b = (char *)ibip_scratch(ctx, SC_LIST, std::max(o.gl, z.lists + z.tables));
+    // the two bit planes are those of the one-CTA loop
+    m.fresh = ibip_scratch(ctx, SC_AVAIL, std::max(o.plane, z.bits));
+    m.root_bits = ibip_scratch(ctx, SC_ADDED, std::max(o.plane, z.bits));
+    m.plane = ibip_scratch(ctx, SC_FB, std::max(o.fb, z.plane));
+    m.values = ibip_scratch(ctx, SC_PRES, z.values);
+    constexpr size_t kCtl = (sizeof(FloodCtl) + 255) / 256 * 256;
+    char *c = (char *)ibip_scratch(ctx, SC_FLOOD, kCtl + sizeof(Flood));
+    int64_t *small = (int64_t *)ibip_scratch(ctx, SC_SMALL, kSmallBytes);
+    if (!m.state || !m.claim || !a || !b || !m.plane || !m.fresh || !m.root_bits || !m.values || !c || !small) return IBIP_ERR_OOM;
+    m.log = a;
+    m.tables2 = a + z.log;
+    m.lists = b;
+    m.tables = b + z.lists;
+    m.ctl = c;
+    m.out = small + 8;
+    Flood f;
+    ibip_flood_fill(&f, dt2, d, inlet, mask, resume, k0, max_steps, seq, step_r2, step_centre, cap, maxd, npore, z, m);
+    f.cancel = ctx->d_cancel;
+    int32_t *keep = nullptr;
+    if (resume) {   // in case the run gives up
+        keep = (int32_t *)ibip_scratch(ctx, SC_MM, (size_t)N * sizeof(int32_t));
+        if (!keep) return IBIP_ERR_OOM;
+        cudaMemcpyAsync(keep, seq, (size_t)N * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
+    }
+    cudaMemsetAsync(m.ctl, 0, sizeof(FloodCtl), s);
+    ibip_prof_end(ctx, IBIP_K_RANK);
+    ibip_prof_begin(ctx, IBIP_K_INVADE);
+    const bool grid = !ctx->no_coop && !ctx->stream_inv && N >= kFloodGridVox;
+    if (!grid) cudaMemcpyAsync(c + kCtl, &f, sizeof(Flood), cudaMemcpyHostToDevice, s);
+    if (ctx->stream_inv) {
+        // server slot: on the high-priority stream, after everything queued
+        // so far on the slot's own stream
+        if (cudaEventRecord(ctx->ev_inv, s) != cudaSuccess ||
+            cudaStreamWaitEvent(ctx->stream_inv, ctx->ev_inv, 0) != cudaSuccess)
+            return ibip_cuda_status(cudaGetLastError());
+        s = ctx->stream_inv;
+    }
+    const int st = grid ? ibip_flood_launch_grid(ctx, f, s)
+                        : ibip_flood_launch_clusters(ctx, (const Flood *)(c + kCtl), 1, maxd, kFloodCluster, s);
+    if (st) return st;
+    ibip_prof_end(ctx, IBIP_K_INVADE);
+    int64_t *ho = (int64_t *)ctx->h_pinned;
+    cudaMemcpyAsync(ho, m.out, 6 * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    const cudaError_t e = ibip_sync(ctx, s);
+    if (e != cudaSuccess) return ibip_cuda_status(e);
+    if (ho[1] == kFloodGiveUp) {
+        ibip_prof_begin(ctx, IBIP_K_RANK);
+        if (resume) cudaMemcpyAsync(seq, keep, (size_t)N * sizeof(int32_t), cudaMemcpyDeviceToDevice, ctx->stream);
+        return kFloodGiveUp;
+    }
+    for (int i = 0; i < kNOut; i++) h_out[i] = 0;
+    h_out[0] = ho[0];
+    h_out[1] = ho[1];
+    h_out[2] = ho[2];
+#ifdef IBIP_CHECKED
+    h_out[kErrSlot] = ho[4];
+    h_out[kErrSlot + 1] = ho[5];
+#endif
+    if (h_out[1] == IBIP_ERR_CANCELLED && ctx->h_cancel) *ctx->h_cancel = 0;   // the request is served
+    return IBIP_OK;
+}
+
 }  // namespace
 
 int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps,
@@ -2050,6 +2134,11 @@ int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, i
         h_out[0] = k0;
         h_out[1] = IBIP_OK;
         return ibip_cuda_status(ibip_sync(ctx, s));
+    }
+    if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf)) {
+        const int st = flood_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, mask, resume,
+                                 k0, h_out);
+        if (st != kFloodGiveUp) return st;
     }
     const JobSizes z = job_sizes(d, npore);
     JobMem mem;

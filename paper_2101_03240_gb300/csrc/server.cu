@@ -135,7 +135,7 @@ extern "C" int64_t ibip_job_footprint(ibip_dims d, int with_dt2)
     add(8 * N);                                                  // (idx, dt2) by rank
     add((int64_t)d.nx * d.ny * ((d.nz + 31) / 32) * 4);          // available bit-plane
     add((int64_t)d.nx * d.ny * ((d.nz + 31) / 32) * 4);          // queued bit-plane
-    add((nl0 + nl1 + nl2 + nl3) * 8);                            // frontier bitmap
+    add((nl0 + nl1 + nl2 + nl3) * 8 + 16);                       // frontier bitmap, or record plane
     add(8 * N + 64);                                             // overflow work lists
     const int64_t maxd = (int64_t)(d.nx - 1) * (d.nx - 1) + (int64_t)(d.ny - 1) * (d.ny - 1) +
                          (int64_t)(d.nz - 1) * (d.nz - 1);
@@ -146,6 +146,7 @@ extern "C" int64_t ibip_job_footprint(ibip_dims d, int with_dt2)
     int64_t nscan = mat > maxd + 2 ? mat : maxd + 2;
     if (N + 2 > nscan) nscan = N + 2;
     for (int q = 0; q < 3; q++) add(scan_work_bytes(nscan));     // scan work, regrown at most thrice
+    add(1 << 21);   // constant parts of the phase tables, which otherwise fit the entries above
     // trapping: widest-path field, tile lists and round counters
     add(4 * N);
     const int64_t nt = (int64_t)((d.nx + 3) / 4) * ((d.ny + 7) / 8) * ((d.nz + 31) / 32);
