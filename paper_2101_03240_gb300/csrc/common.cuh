@@ -29,13 +29,12 @@ enum ScratchSlot {
     SC_LIST,      // int32 overflow work lists of the invasion kernel
     SC_FL,        // uint8 first opening level per voxel, and the level radii
     SC_BSTAT,     // batched invasion: per-image pore statistics
-    SC_BARENA,    // batched invasion: per-image ranks, bit-planes, bitmaps
+    SC_BARENA,    // batched invasion: per-image tables
     SC_BJOBS,     // batched invasion: job table
     SC_BDT2,      // batched invasion: EDTs of images given without one
     SC_LIT,       // paper-literal invasion: bucket lists, counters, bit-plane
     SC_LITB,      // batched paper-literal invasion: every image's buckets, lists, bit-planes
     SC_LITJ,      // batched paper-literal invasion: job table, statistics, outputs
-    SC_BSORT,     // batched invasion: sort job table, presence pool
     SC_FLOOD,     // invasion by value phases: counters, job table
     SC_NSLOTS
 };

@@ -981,7 +981,8 @@ __device__ void flood_body(const Flood &f, const int T, const int c)
         if (steps >= f.max_steps) { status = IBIP_ERR_STEP_LIMIT; break; }
         n_phases++;
         ph.pbase = pbase;
-        ph.chunk = ph.R >= 16384 ? 32 : ph.R >= 64 ? 8 : 16;
+        // log slots a warp or CTA takes at a time: unused ones stay few
+        ph.chunk = max(2, min(16, ph.R / (4 * GW)));
         bool planes = false;    // the bit planes hold this phase
         bool dropped = false;   // some groups of this phase were run again
         for (ph.round = 0;; ph.round++) {
@@ -1128,9 +1129,10 @@ __device__ void flood_body(const Flood &f, const int T, const int c)
                     __stcg(f.cur + i, 0u);
                 } else {
                     __stcg(f.cur + r, id);
-                    if (d & 2) ctl->longs = 1;
+                    if ((d & 3) == 3) ctl->longs = 1;
+                    // flags: 1 a CTA, 3 a CTA with the planes
                     if ((d & 1) || ph.t >= 9)
-                        __stcg(f.todo + f.root_cap - 1 - atomicAdd(&ctl->todoC, 1), (d & 2) ? ~r : r);
+                        __stcg(f.todo + f.root_cap - 1 - atomicAdd(&ctl->todoC, 1), (d & 3) == 3 ? ~r : r);
                     else __stcg(f.todo + atomicAdd(&ctl->todoW, 1), r);
                 }
             }
@@ -1185,7 +1187,7 @@ __device__ void flood_body(const Flood &f, const int T, const int c)
                 if (e.x < 0 || !in_range(f.ctl, e.x, (int64_t)f.nx * f.ny * f.nz, P_LOG)) continue;
                 if (lane == 0) {
                     mine++;
-                    if (huge && f.dt2[e.x] >= kHuge) __stcg(f.todo + atomicAdd(&ctl->huge, 1), i);
+                    if (huge && f.dt2[e.x] >= kHuge) { const int at = atomicAdd(&ctl->huge, 1); if (at < f.root_cap) __stcg(f.todo + at, i); }
                 }
                 if (!(e.z & kLast)) continue;
                 int s = 0;
@@ -1203,7 +1205,7 @@ __device__ void flood_body(const Flood &f, const int T, const int c)
                 const int4 e = __ldcg(f.log + i);
                 if (e.x < 0 || !in_range(f.ctl, e.x, (int64_t)f.nx * f.ny * f.nz, P_LOG)) continue;
                 mine++;
-                if (huge && f.dt2[e.x] >= kHuge) __stcg(f.todo + atomicAdd(&ctl->huge, 1), i);
+                if (huge && f.dt2[e.x] >= kHuge) { const int at = atomicAdd(&ctl->huge, 1); if (at < f.root_cap) __stcg(f.todo + at, i); }
                 if (!(e.z & kLast)) continue;
                 atomicOr(f.plane + (e.y >> 5), 1u << (e.y & 31));
                 __stcg(f.claim + e.y, (u32)((e.z & ~kLast) + 1));
@@ -1279,6 +1281,7 @@ __device__ void flood_body(const Flood &f, const int T, const int c)
         // `per` log entries, single voxels by lanes, balls by the whole warp
         if (c == 0 && tid == 0) ctl->R = 0;
         const int nhuge = huge ? __ldcg(&ctl->huge) : 0;
+        if (nhuge > f.root_cap) { status = kFloodGiveUp; break; }
         const int wpe = min(64, max(1, GW / max(nlog, 1)));
         const int per = max(1, min(32, nlog / GW));
         const int unit = gw / wpe, sub = gw % wpe, units = GW / wpe;
@@ -1406,7 +1409,10 @@ FloodSizes ibip_flood_sizes(ibip_dims d, int64_t npore, int maxd)
 {
     FloodSizes z;
     const int64_t N = nvox(d);
-    z.root_cap = z.log_cap = (int)(npore / 4) + 16384;
+    // packs of narrow pores have ~18 % of their pore voxels as roots of the
+    // last phase, and log some steps again in every round
+    z.root_cap = (int)(npore / 4) + 4096;
+    z.log_cap = (int)(npore / 2) + 16384;
     z.state = up256(((size_t)N + 8) * 2);
     z.claim = up256(((size_t)N + 4) * 4);
     z.bits = up256((size_t)d.nx * d.ny * ((d.nz + 31) / 32) * 4);
@@ -1454,8 +1460,10 @@ void ibip_flood_fill(Flood *f, const int32_t *dt2, ibip_dims d, int inlet, const
     f->out = m.out;
     f->cancel = nullptr;
     f->rec = nullptr;
-    // a group longer than this is a serial chain that the one-CTA loop runs faster
-    f->budget = (int)std::min<int64_t>(std::max<int64_t>(N / 1024, 1024), 1 << 17);
+    // A group longer than this is a serial chain that the one-CTA loop runs
+    // faster: a long group takes ~2 us a step, the loop 0.3-0.4 us a step on
+    // all the steps, of which there is one for 15-25 voxels.
+    f->budget = (int)std::min<int64_t>(std::max<int64_t>(N / 64, 4096), 1 << 18);
 }
 
 int ibip_flood_launch_grid(ibip_ctx *ctx, const Flood &f, cudaStream_t s)

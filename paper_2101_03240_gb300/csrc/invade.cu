@@ -43,8 +43,16 @@ constexpr int kNT = 768;         // threads of the persistent CTA (measured: 384
 constexpr int kChunk = 4096;     // voxels per rank-sort chunk (minimum)
 constexpr int kSmemL1Max = 12288;   // level-1 words of one image of a batched call (shared memory)
 constexpr int kNOut = kInvStats;   // int64 outputs of the invasion kernel
-constexpr int64_t kFloodGridVox = 1 << 21;   // images from this size on run by phases on the whole GPU
-constexpr int kFloodCluster = 16;            // CTAs of one image otherwise
+// Images from this size on run by phases on the whole GPU, smaller ones on
+// one cluster, whose barrier is cheaper (blobs / pack, cluster of 16 against
+// the whole GPU: 64^3 3.2 / 3.6 against 3.5 / 3.7 ms, 96^3 5.5 / 5.9 against
+// 5.1 / 5.6 ms; the line is the middle).
+constexpr int64_t kFloodGridVox = 1 << 19;
+constexpr int kFloodCluster = 16;   // CTAs of one image on a cluster
+// CTAs of each image of a batch of n: fewer when the images fill the GPU
+// (96 images of 32^3-160^3, invasion only: clusters of 1, 2, 4, 8, 16 take
+// 185, 103, 68, 54, 86 ms).
+int flood_batch_cluster(int n) { return n <= 24 ? 16 : n <= 128 ? 8 : 4; }
 static_assert(64 + kNOut * sizeof(long long) <= kSmallBytes, "output slot too small");
 
 typedef unsigned long long u64;
@@ -175,54 +183,7 @@ __global__ void k_last_bucket_rank(const int32_t *pos, int base, int64_t *out)
     if (threadIdx.x == 0) *out = (int64_t)(*pos - base);
 }
 
-// ------------------------------------------- rank sort of many images --
-// The same counting sort for every image of a batch at once: per-image
-// arrays live at offsets in pooled buffers, one flat scan serves all images
-// (each subtracts the pool's running total at its own start), and each
-// kernel finds its image from its block index by binary search over the
-// images' first blocks.
-struct SortJob {
-    const int32_t *dt2;
-    int64_t N;
-    int32_t *seq, *rank;
-    int2 *okey;
-    int64_t pres_off;   // first entry of this image's presence segment
-    int maxd, hasinf;
-    int pres_base;      // pool total before the segment (device-written)
-    int B;              // distinct values (device-written, then read back)
-    int S, C, smem;     // chunk length, chunks, counters in shared memory
-    int64_t mat_off;    // first entry of this image's (bucket, chunk) matrix
-    int mat_base;       // pool total before the matrix (device-written)
-    int blk_vox, blk_chunk;   // first block of this image in the voxel / chunk launches
-    int64_t *out;             // the invasion's output slots (the last bucket's first rank goes there)
-};
-
-__device__ __forceinline__ int find_job(const SortJob *jobs, int n, int blk, bool chunk)
-{
-    int lo = 0, hi = n;   // largest j whose first block is <= blk
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if ((chunk ? jobs[mid].blk_chunk : jobs[mid].blk_vox) <= blk) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
 constexpr int kVoxBlock = 256, kVoxPer = 8;   // voxel launches: 2048 voxels per block
-
-// seq = -1 on pore, 0 on solid; presence of each finite value
-__global__ void k_seq_pres_b(const SortJob *__restrict__ jobs, int n, int32_t *pres)
-{
-    const int j = find_job(jobs, n, blockIdx.x, false);
-    const SortJob &J = jobs[j];
-    const int64_t v0 = (int64_t)(blockIdx.x - J.blk_vox) * kVoxBlock * kVoxPer;
-    for (int q = 0; q < kVoxPer; q++) {
-        const int64_t v = v0 + q * kVoxBlock + threadIdx.x;
-        if (v >= J.N) break;
-        const int d = J.dt2[v];
-        J.seq[v] = d > 0 ? -1 : 0;
-        if (d > 0 && d != IBIP_INF32) pres[J.pres_off + d] = 1;
-    }
-}
 
 // pore statistics of many images (as k_stats), kVoxBlock * kVoxPer voxels
 // per block; a block finds its image by binary search over first blocks
@@ -258,106 +219,6 @@ __global__ void k_stats_b(const StatJob *__restrict__ jobs, int n, int *stats)
         atomicMax(stats + 3 * lo, mx);
         atomicAdd(stats + 3 * lo + 1, np);
         atomicOr(stats + 3 * lo + 2, inf);
-    }
-}
-
-// after the flat inclusive scan of the presence pool: each image's base and
-// number of distinct values
-__global__ void k_pres_base_b(SortJob *jobs, int n, const int32_t *__restrict__ incl)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    SortJob &J = jobs[j];
-    const int base = J.pres_off > 0 ? incl[J.pres_off - 1] : 0;
-    J.pres_base = base;
-    J.B = J.hasinf ? 1 : incl[J.pres_off + J.maxd] - base;
-}
-
-__device__ __forceinline__ int bucket_b(const SortJob &J, const int32_t *__restrict__ incl, int d)
-{
-    if (d <= 0) return -1;
-    if (J.hasinf) return 0;
-    return J.B - (__ldg(incl + J.pres_off + d) - J.pres_base);
-}
-
-// k_chunk_hist for every image: one warp per chunk
-__global__ void k_chunk_hist_b(const SortJob *__restrict__ jobs, int n, const int32_t *__restrict__ incl,
-                               int32_t *mat)
-{
-    extern __shared__ int32_t s_cnt[];
-    const int j = find_job(jobs, n, blockIdx.x, true);
-    const SortJob &J = jobs[j];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int c = (blockIdx.x - J.blk_chunk) * (blockDim.x >> 5) + w;
-    if (c >= J.C) return;
-    int32_t *m = mat + J.mat_off;
-    int32_t *cnt = J.smem ? s_cnt + w * J.B : nullptr;
-    for (int b = lane; b < J.B; b += 32) {
-        if (J.smem) cnt[b] = 0; else m[(int64_t)b * J.C + c] = 0;
-    }
-    __syncwarp();
-    const int64_t v0 = (int64_t)c * J.S, v1 = min(J.N, v0 + J.S);
-    for (int64_t v = v0 + lane; v - lane < v1; v += 32) {
-        const int b = v < v1 ? bucket_b(J, incl, J.dt2[v]) : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, b);
-        const int leader = __ffs(peers) - 1;
-        if (lane == leader && b >= 0) {
-            if (J.smem) cnt[b] += __popc(peers);
-            else m[(int64_t)b * J.C + c] += __popc(peers);
-        }
-        __syncwarp();
-    }
-    if (J.smem)
-        for (int b = lane; b < J.B; b += 32) m[(int64_t)b * J.C + c] = cnt[b];
-}
-
-// after the flat exclusive scan of the matrix pool: each image's base
-__global__ void k_mat_base_b(SortJob *jobs, int n, const int32_t *__restrict__ mat)
-{
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    SortJob &J = jobs[j];
-    J.mat_base = mat[J.mat_off];
-    J.out[kFirst1Slot] = (int64_t)(mat[J.mat_off + (int64_t)(J.B - 1) * J.C] - J.mat_base);
-}
-
-__global__ void k_chunk_scatter_b(const SortJob *__restrict__ jobs, int n, const int32_t *__restrict__ incl,
-                                  int32_t *mat)
-{
-    extern __shared__ int32_t s_cnt[];
-    const int j = find_job(jobs, n, blockIdx.x, true);
-    const SortJob &J = jobs[j];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int c = (blockIdx.x - J.blk_chunk) * (blockDim.x >> 5) + w;
-    if (c >= J.C) return;
-    int32_t *m = mat + J.mat_off;
-    int32_t *cnt = J.smem ? s_cnt + w * J.B : nullptr;
-    if (J.smem) {
-        for (int b = lane; b < J.B; b += 32) cnt[b] = m[(int64_t)b * J.C + c] - J.mat_base;
-        __syncwarp();
-    }
-    const int64_t v0 = (int64_t)c * J.S, v1 = min(J.N, v0 + J.S);
-    const unsigned lt = (1u << lane) - 1;
-    for (int64_t v = v0 + lane; v - lane < v1; v += 32) {
-        const int d = v < v1 ? J.dt2[v] : 0;
-        const int b = v < v1 ? bucket_b(J, incl, d) : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, b);
-        const int leader = __ffs(peers) - 1;
-        int base = 0;
-        if (lane == leader && b >= 0) base = J.smem ? cnt[b] : m[(int64_t)b * J.C + c] - J.mat_base;
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (b >= 0) {
-            const int r = base + __popc(peers & lt);
-            J.rank[v] = r;
-            J.okey[r] = make_int2((int)v, d);
-        } else if (v < v1) {
-            J.rank[v] = -1;
-        }
-        if (lane == leader && b >= 0) {
-            if (J.smem) cnt[b] = base + __popc(peers);
-            else m[(int64_t)b * J.C + c] = base + __popc(peers) + J.mat_base;
-        }
-        __syncwarp();
     }
 }
 
@@ -1790,47 +1651,6 @@ __global__ void __launch_bounds__(kNT, 1) k_invade(Inv a, FastDiv fd_nyz, FastDi
     invade_body<L1SMEM, PROF>(a, fd_nyz, fd_nz, gC, gD);
 }
 
-// One image per CTA: many invasions in one launch (all with level 1 of the
-// rank bitmap in shared memory).
-struct InvJob {
-    Inv a;
-    FastDiv fd_nyz, fd_nz;
-    int *gC, *gD;
-    int blk_plane;   // first block of this image in the batched plane set-up
-    int flag;        // this image's completion record
-};
-
-// bit-planes and first candidates of every image: one thread per word
-__global__ void k_plane_init_b(const InvJob *__restrict__ jobs, int n)
-{
-    int lo = 0, hi = n;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (jobs[mid].blk_plane <= (int)blockIdx.x) lo = mid; else hi = mid;
-    }
-    const Inv &a = jobs[lo].a;
-    const int64_t w = (int64_t)(blockIdx.x - jobs[lo].blk_plane) * blockDim.x + threadIdx.x;
-    if (w < (int64_t)a.nx * a.ny * a.NW) plane_word(a, w);
-}
-
-// rec (host-mapped, when given): image i's steps and status, then its done
-// flag, once its results are visible to later kernels on the device.
-__global__ void __launch_bounds__(kNT, 1) k_invade_batch(const InvJob *__restrict__ jobs, IbipBatchDone *rec)
-{
-    const InvJob j = jobs[blockIdx.x];
-    invade_body<true, false>(j.a, j.fd_nyz, j.fd_nz, j.gC, j.gD);
-    if (!rec) return;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile IbipBatchDone *r = rec + j.flag;
-        r->steps = j.a.out[0];
-        r->status = (int32_t)j.a.out[1];
-        __threadfence_system();
-        r->done = 1;
-    }
-}
-
 }  // namespace
 
 // --------------------------------------------------------------- launcher --
@@ -1882,19 +1702,6 @@ JobSizes job_sizes(ibip_dims d, int npore)
     z.gl = up256((size_t)2 * npore * sizeof(int) + 64);
     z.out = up256(kNOut * sizeof(int64_t));
     return z;
-}
-
-JobMem carve(char *p, const JobSizes &z)
-{
-    JobMem m;
-    m.rank = (int32_t *)p; p += z.rank;
-    m.okey = (int2 *)p; p += z.okey;
-    m.avail = (uint32_t *)p; p += z.plane;
-    m.added = (uint32_t *)p; p += z.plane;
-    m.fb = (u64 *)p; p += z.fb;
-    m.gl = (int *)p; p += z.gl;
-    m.out = (int64_t *)p;
-    return m;
 }
 
 // The invasion kernel's view of one image, its scratch carved as in `mem`.
@@ -2025,7 +1832,8 @@ bool l1_fits_smem(const Inv &a)
 // thread-block cluster.  kFloodGiveUp: the run outgrew its tables and the
 // one-CTA loop has to take the image from the start (a resumed run cannot:
 // its sequence image is partly written by then, so it is copied back first).
-// The tables share the scratch slots of that loop and of the EDT passes.
+// The tables share the scratch slots of that loop, of the EDT passes and of
+// the widest path, none of which runs meanwhile.
 int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps, int32_t *seq,
               int32_t *step_r2, int32_t *step_centre, int64_t cap, int maxd, int npore, const uint8_t *mask, int resume,
               int64_t k0, int64_t *h_out)
@@ -2037,7 +1845,8 @@ int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t
     FloodMem m;
     m.state = ibip_scratch(ctx, SC_D1, z.state);
     m.claim = ibip_scratch(ctx, SC_RANK, std::max(o.rank, z.claim));
-    char *a = (char *)ibip_scratch(ctx, SC_OKEY, std::max(o.okey, z.log + z.tables2));
+    m.log = ibip_scratch(ctx, SC_OKEY, std::max(o.okey, z.log));
+    m.tables2 = ibip_scratch(ctx, SC_MM, std::max((size_t)N * 4, z.tables2));
     char *b = (char *)ibip_scratch(ctx, SC_LIST, std::max(o.gl, z.lists + z.tables));
     // the two bit planes are those of the one-CTA loop
     m.fresh = ibip_scratch(ctx, SC_AVAIL, std::max(o.plane, z.bits));
@@ -2047,9 +1856,7 @@ int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t
     constexpr size_t kCtl = (sizeof(FloodCtl) + 255) / 256 * 256;
     char *c = (char *)ibip_scratch(ctx, SC_FLOOD, kCtl + sizeof(Flood));
     int64_t *small = (int64_t *)ibip_scratch(ctx, SC_SMALL, kSmallBytes);
-    if (!m.state || !m.claim || !a || !b || !m.plane || !m.fresh || !m.root_bits || !m.values || !c || !small) return IBIP_ERR_OOM;
-    m.log = a;
-    m.tables2 = a + z.log;
+    if (!m.state || !m.claim || !m.log || !m.tables2 || !b || !m.plane || !m.fresh || !m.root_bits || !m.values || !c || !small) return IBIP_ERR_OOM;
     m.lists = b;
     m.tables = b + z.lists;
     m.ctl = c;
@@ -2059,7 +1866,7 @@ int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t
     f.cancel = ctx->d_cancel;
     int32_t *keep = nullptr;
     if (resume) {   // in case the run gives up
-        keep = (int32_t *)ibip_scratch(ctx, SC_MM, (size_t)N * sizeof(int32_t));
+        keep = (int32_t *)ibip_scratch(ctx, SC_G2, (size_t)N * sizeof(int32_t));
         if (!keep) return IBIP_ERR_OOM;
         cudaMemcpyAsync(keep, seq, (size_t)N * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
     }
@@ -2101,45 +1908,13 @@ int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t
     return IBIP_OK;
 }
 
-}  // namespace
-
-int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps,
-                    int32_t *seq, int32_t *step_r2, int32_t *step_centre, int64_t cap, int64_t *h_out,
-                    const uint8_t *mask, int resume)
+// The one-CTA loop: what the phases do not take (no solid, large values,
+// traced runs) or gave up.
+int loop_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps, int32_t *seq,
+             int32_t *step_r2, int32_t *step_centre, int64_t cap, int maxd, int npore, int hasinf, const uint8_t *mask,
+             int resume, int64_t k0, int64_t *h_out)
 {
     cudaStream_t s = ctx->stream;
-    const int64_t N = nvox(d);
-    int k0 = 0;   // steps of the run being resumed: the largest seq value
-    if (resume) {
-        int st = ibip_max_launch(ctx, seq, N, &k0);
-        if (st) return st;
-    }
-    int *stats = (int *)ibip_scratch(ctx, SC_SMALL, kSmallBytes);
-    if (!stats) return IBIP_ERR_OOM;
-    int *h = (int *)ctx->h_pinned;
-    ibip_prof_begin(ctx, IBIP_K_RANK);
-    cudaMemsetAsync(stats, 0, 3 * sizeof(int), s);
-    k_stats<<<ctx->sm_count * 8, 256, 0, s>>>(dt2, N, stats);
-    IBIP_LAUNCH(ctx);
-    cudaMemcpyAsync(h, stats, 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (ibip_sync(ctx, s) != cudaSuccess) return IBIP_ERR_CUDA;
-    const int maxd = h[0], npore = h[1], hasinf = h[2];
-    if (npore == 0) {
-        if (!resume) {
-            k_seq_init<<<ctx->sm_count * 8, 256, 0, s>>>(dt2, N, seq);
-            IBIP_LAUNCH(ctx);
-        }
-        ibip_prof_end(ctx, IBIP_K_RANK);
-        for (int i = 0; i < kNOut; i++) h_out[i] = 0;
-        h_out[0] = k0;
-        h_out[1] = IBIP_OK;
-        return ibip_cuda_status(ibip_sync(ctx, s));
-    }
-    if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf)) {
-        const int st = flood_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, mask, resume,
-                                 k0, h_out);
-        if (st != kFloodGiveUp) return st;
-    }
     const JobSizes z = job_sizes(d, npore);
     JobMem mem;
     mem.rank = (int32_t *)ibip_scratch(ctx, SC_RANK, z.rank);
@@ -2200,6 +1975,49 @@ int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, i
     return IBIP_OK;
 }
 
+}  // namespace
+
+int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps,
+                    int32_t *seq, int32_t *step_r2, int32_t *step_centre, int64_t cap, int64_t *h_out,
+                    const uint8_t *mask, int resume)
+{
+    cudaStream_t s = ctx->stream;
+    const int64_t N = nvox(d);
+    int k0 = 0;   // steps of the run being resumed: the largest seq value
+    if (resume) {
+        int st = ibip_max_launch(ctx, seq, N, &k0);
+        if (st) return st;
+    }
+    int *stats = (int *)ibip_scratch(ctx, SC_SMALL, kSmallBytes);
+    if (!stats) return IBIP_ERR_OOM;
+    int *h = (int *)ctx->h_pinned;
+    ibip_prof_begin(ctx, IBIP_K_RANK);
+    cudaMemsetAsync(stats, 0, 3 * sizeof(int), s);
+    k_stats<<<ctx->sm_count * 8, 256, 0, s>>>(dt2, N, stats);
+    IBIP_LAUNCH(ctx);
+    cudaMemcpyAsync(h, stats, 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (ibip_sync(ctx, s) != cudaSuccess) return IBIP_ERR_CUDA;
+    const int maxd = h[0], npore = h[1], hasinf = h[2];
+    if (npore == 0) {
+        if (!resume) {
+            k_seq_init<<<ctx->sm_count * 8, 256, 0, s>>>(dt2, N, seq);
+            IBIP_LAUNCH(ctx);
+        }
+        ibip_prof_end(ctx, IBIP_K_RANK);
+        for (int i = 0; i < kNOut; i++) h_out[i] = 0;
+        h_out[0] = k0;
+        h_out[1] = IBIP_OK;
+        return ibip_cuda_status(ibip_sync(ctx, s));
+    }
+    if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf)) {
+        const int st = flood_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, mask, resume,
+                                 k0, h_out);
+        if (st != kFloodGiveUp) return st;
+    }
+    return loop_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, hasinf, mask, resume, k0,
+                    h_out);
+}
+
 int ibip_stats_launch(ibip_ctx *ctx, const int32_t *dt2, int64_t N, int *stats)
 {
     k_stats<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(dt2, N, stats);
@@ -2237,152 +2055,80 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
     if (ibip_sync(ctx, s) != cudaSuccess) return IBIP_ERR_CUDA;
     std::vector<int> maxd(n), npore(n), hasinf(n);
     size_t total = 0;
-    std::vector<JobSizes> z(n);
+    int top = 1;   // largest finite dt2 of the images run by phases
+    std::vector<FloodSizes> z(n);
+    std::vector<int> idx, single;   // images run by phases, and by the one-CTA loop
+    int64_t pore_total = 0;
     for (int j = 0; j < n; j++) {
         maxd[j] = h[3 * j]; npore[j] = h[3 * j + 1]; hasinf[j] = h[3 * j + 2];
         it[j].n_steps = 0;
         it[j].status = IBIP_OK;
         if (npore[j] == 0) continue;
-        z[j] = job_sizes(it[j].d, npore[j]);
-        if ((npore[j] + 63) / 64 > (int64_t)kSmemL1Max * 64) return IBIP_ERR_ARG;   // too large for one-CTA batching
-        total += z[j].total();
-    }
-    char *arena = (char *)ibip_scratch(ctx, SC_BARENA, total + 256);
-    if (!arena) return IBIP_ERR_OOM;
-    std::vector<InvJob> jobs;
-    std::vector<int> idx;
-    std::vector<int64_t *> outs(n, nullptr);
-    size_t off = 0, dyn = 0;
-    // images with pore: one sort job each; the others only need seq
-    std::vector<SortJob> sj;
-    std::vector<JobMem> mems;
-    int64_t pres_total = 0, pore_total = 0;
-    int blk_vox = 0;
-    for (int j = 0; j < n; j++) {
-        if (npore[j] == 0) {
-            k_seq_init<<<ctx->sm_count * 2, 256, 0, s>>>(it[j].dt2, nvox(it[j].d), it[j].seq);
-            IBIP_LAUNCH(ctx);
-            continue;
-        }
+        if ((npore[j] + 63) / 64 > (int64_t)kSmemL1Max * 64) return IBIP_ERR_ARG;   // too large for a batch
         pore_total += npore[j];
-        if (pore_total >= (1ll << 31)) return IBIP_ERR_ARG;   // the whole batch's ranks share one int32 scan
-        const JobMem mem = carve(arena + off, z[j]);
-        off += z[j].total();
-        SortJob q = {};
-        q.dt2 = it[j].dt2; q.N = nvox(it[j].d); q.seq = it[j].seq; q.rank = mem.rank; q.okey = mem.okey;
-        q.out = mem.out;
-        q.maxd = hasinf[j] ? 0 : maxd[j]; q.hasinf = hasinf[j];
-        q.pres_off = pres_total;
-        pres_total += (int64_t)q.maxd + 1;
-        q.blk_vox = blk_vox;
-        blk_vox += (int)((q.N + kVoxBlock * kVoxPer - 1) / (kVoxBlock * kVoxPer));
-        sj.push_back(q);
-        mems.push_back(mem);
+        if (pore_total >= (1ll << 31)) return IBIP_ERR_ARG;
+        if (!ibip_flood_ok(it[j].d, npore[j], maxd[j], hasinf[j])) { single.push_back(j); continue; }
+        z[j] = ibip_flood_sizes(it[j].d, npore[j], maxd[j]);
+        total += z[j].total();
+        top = std::max(top, maxd[j]);
         idx.push_back(j);
     }
-    const int m0 = (int)sj.size();
-    if (m0 > 0) {
-        // presence of every value: one scan and one read-back for all images
-        const size_t tab = ((size_t)m0 * sizeof(SortJob) + 255) / 256 * 256;
-        char *sw = (char *)ibip_scratch(ctx, SC_BSORT, tab + (size_t)pres_total * 4);
-        if (!sw) return IBIP_ERR_OOM;
-        SortJob *djobs = (SortJob *)sw;
-        int32_t *pres = (int32_t *)(sw + tab);
-        cudaMemcpyAsync(djobs, sj.data(), (size_t)m0 * sizeof(SortJob), cudaMemcpyHostToDevice, s);
-        cudaMemsetAsync(pres, 0, (size_t)pres_total * 4, s);
-        k_seq_pres_b<<<blk_vox, kVoxBlock, 0, s>>>(djobs, m0, pres);
-        IBIP_LAUNCH(ctx);
-        int st = ibip_scan_incl_i32(ctx, pres, pres, pres_total);
-        if (st) return st;
-        k_pres_base_b<<<(m0 + 127) / 128, 128, 0, s>>>(djobs, m0, pres);
-        IBIP_LAUNCH(ctx);
-        cudaMemcpyAsync(sj.data(), djobs, (size_t)m0 * sizeof(SortJob), cudaMemcpyDeviceToHost, s);
-        if (ibip_sync(ctx, s) != cudaSuccess) return IBIP_ERR_CUDA;
-        // chunking of each image's counting sort, as in the one-image set-up
-        const int wpb = 4;
-        int64_t mat_total = 0;
-        int blk_chunk = 0, maxBs = 1;
-        for (auto &q : sj) {
-            int64_t S = kChunk;
-            const int64_t mat_lim = std::max(q.N / 4, (int64_t)1 << 20);
-            while (S < q.N && (q.N + S - 1) / S * (int64_t)q.B > mat_lim) S *= 2;
-            q.S = (int)S;
-            q.C = (int)((q.N + S - 1) / S);
-            q.smem = q.B <= 1024;
-            if (q.smem) maxBs = std::max(maxBs, q.B);
-            q.mat_off = mat_total;
-            mat_total += (int64_t)q.C * q.B;
-            q.blk_chunk = blk_chunk;
-            blk_chunk += (q.C + wpb - 1) / wpb;
-        }
-        if (mat_total >= (1ll << 31)) return IBIP_ERR_ARG;
-        int32_t *mat = (int32_t *)ibip_scratch(ctx, SC_MAT, (size_t)mat_total * sizeof(int32_t));
-        if (!mat) return IBIP_ERR_OOM;
-        cudaMemcpyAsync(djobs, sj.data(), (size_t)m0 * sizeof(SortJob), cudaMemcpyHostToDevice, s);
-        const size_t sm = (size_t)wpb * maxBs * sizeof(int32_t);
-        k_chunk_hist_b<<<blk_chunk, wpb * 32, sm, s>>>(djobs, m0, pres, mat);
-        IBIP_LAUNCH(ctx);
-        st = ibip_scan_excl_i32(ctx, mat, mat, mat_total);
-        if (st) return st;
-        k_mat_base_b<<<(m0 + 127) / 128, 128, 0, s>>>(djobs, m0, mat);
-        IBIP_LAUNCH(ctx);
-        k_chunk_scatter_b<<<blk_chunk, wpb * 32, sm, s>>>(djobs, m0, pres, mat);
+    for (int j = 0; j < n; j++) {
+        if (npore[j]) continue;
+        k_seq_init<<<ctx->sm_count * 2, 256, 0, s>>>(it[j].dt2, nvox(it[j].d), it[j].seq);
         IBIP_LAUNCH(ctx);
     }
-    for (int q = 0; q < m0; q++) {
-        const int j = idx[q];
-        const JobMem &mem = mems[q];
-        InvJob J;
-        J.a = make_inv(it[j].dt2, it[j].d, it[j].inlet, it[j].max_steps, it[j].seq, it[j].step_r2, it[j].step_centre,
-                       it[j].cap, maxd[j], npore[j], mem, nullptr, 0, 0);
-        J.a.cancel = ctx->d_cancel;
-        cudaMemsetAsync(mem.fb, 0, fb_words(J.a) * sizeof(u64), s);
-        J.fd_nyz = make_fastdiv((uint32_t)it[j].d.ny * (uint32_t)it[j].d.nz);
-        J.fd_nz = make_fastdiv((uint32_t)it[j].d.nz);
-        J.gC = mem.gl;
-        J.gD = mem.gl + npore[j];
-        J.blk_plane = 0;
-        dyn = std::max(dyn, invade_dyn_smem(J.a, true));
-        outs[j] = mem.out;
-        jobs.push_back(J);
-    }
-    const int m = (int)jobs.size();
+    const int m = (int)idx.size();
+    int first_err = IBIP_OK;
     if (m > 0) {
-        std::vector<int> order(m);
-        for (int q = 0; q < m; q++) order[q] = q;
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-            return nvox(it[idx[a]].d) > nvox(it[idx[b]].d);
-        });
-        std::vector<InvJob> sorted(m);
-        int blk_plane = 0;
-        for (int q = 0; q < m; q++) {
-            sorted[q] = jobs[order[q]];
-            sorted[q].flag = order[q];
-            sorted[q].blk_plane = blk_plane;
-            const Inv &a = sorted[q].a;
-            blk_plane += (int)(((int64_t)a.nx * a.ny * a.NW + 255) / 256);
-        }
-        InvJob *djobs = (InvJob *)ibip_scratch(ctx, SC_BJOBS, (size_t)m * sizeof(InvJob));
-        if (!djobs) return IBIP_ERR_OOM;
-        cudaMemcpyAsync(djobs, sorted.data(), (size_t)m * sizeof(InvJob), cudaMemcpyHostToDevice, s);
-        k_plane_init_b<<<blk_plane, 256, 0, s>>>(djobs, m);
-        IBIP_LAUNCH(ctx);
-        ibip_prof_end(ctx, IBIP_K_RANK);
-        ibip_prof_begin(ctx, IBIP_K_INVADE);
-        allow_max_dyn_smem((const void *)k_invade_batch);
+        // largest first, so that the long runs start at once
+        std::stable_sort(idx.begin(), idx.end(), [&](int a, int b) { return nvox(it[a].d) > nvox(it[b].d); });
+        constexpr size_t kCtl = (sizeof(FloodCtl) + 255) / 256 * 256, kOut = 64;
+        char *arena = (char *)ibip_scratch(ctx, SC_BARENA, total + 256);
+        char *tab = (char *)ibip_scratch(ctx, SC_BJOBS, (size_t)m * (kCtl + kOut + sizeof(Flood)));
+        if (!arena || !tab) return IBIP_ERR_OOM;
+        char *outs = tab + (size_t)m * kCtl;
+        Flood *djobs = (Flood *)(outs + (size_t)m * kOut);
         volatile IbipBatchDone *hd = early ? (volatile IbipBatchDone *)ctx->h_done : nullptr;
+        std::vector<Flood> jobs(m);
+        char *p = arena;
+        auto take = [&](size_t b) { char *r = p; p += b; return (void *)r; };
+        for (int q = 0; q < m; q++) {
+            const int j = idx[q];
+            FloodMem mem;
+            mem.state = take(z[j].state);
+            mem.claim = take(z[j].claim);
+            mem.plane = take(z[j].plane);
+            mem.fresh = take(z[j].bits);
+            mem.root_bits = take(z[j].bits);
+            mem.lists = take(z[j].lists);
+            mem.tables = take(z[j].tables);
+            mem.tables2 = take(z[j].tables2);
+            mem.log = take(z[j].log);
+            mem.values = take(z[j].values);
+            mem.ctl = tab + (size_t)q * kCtl;
+            mem.out = (int64_t *)(outs + (size_t)q * kOut);
+            ibip_flood_fill(&jobs[q], it[j].dt2, it[j].d, it[j].inlet, nullptr, 0, 0, it[j].max_steps, it[j].seq,
+                            it[j].step_r2, it[j].step_centre, it[j].cap, maxd[j], npore[j], z[j], mem);
+            jobs[q].cancel = ctx->d_cancel;
+            jobs[q].rec = hd ? (IbipBatchDone *)ctx->d_done + q : nullptr;
+        }
+        cudaMemsetAsync(tab, 0, (size_t)m * kCtl, s);
+        cudaMemcpyAsync(djobs, jobs.data(), (size_t)m * sizeof(Flood), cudaMemcpyHostToDevice, s);
         if (hd)
             for (int q = 0; q < m; q++) hd[q].done = 0;
-        k_invade_batch<<<m, kNT, dyn, s>>>(djobs, hd ? (IbipBatchDone *)ctx->d_done : nullptr);
-        IBIP_LAUNCH(ctx);
+        ibip_prof_end(ctx, IBIP_K_RANK);
+        ibip_prof_begin(ctx, IBIP_K_INVADE);
+        const int st = ibip_flood_launch_clusters(ctx, djobs, m, top, flood_batch_cluster(m), s);
+        if (st) return st;
         ibip_prof_end(ctx, IBIP_K_INVADE);
         if (hd) {
-            // records arrive as CTAs finish; once all but kTail images are
+            // records arrive as clusters finish; once all but kTail images are
             // done, `early` post-processes those while the rest still run
             constexpr int kTail = 8;
             std::vector<char> seen(m, 0);
             std::vector<int> done;
-            int nseen = 0, first_err = IBIP_OK;
+            int nseen = 0;
             bool fired = false;
             for (;;) {
                 const bool ended = cudaStreamQuery(s) != cudaErrorNotReady;
@@ -2391,14 +2137,14 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
                     std::atomic_thread_fence(std::memory_order_acquire);   // the record, then its flag
                     seen[q] = 1;
                     nseen++;
+                    if (hd[q].status == kFloodGiveUp) { single.push_back(idx[q]); continue; }
                     it[idx[q]].n_steps = hd[q].steps;
                     it[idx[q]].status = hd[q].status;
                     done.push_back(idx[q]);
                 }
-                if (!fired && nseen > 0 && m - nseen <= kTail && nseen < m) {
+                if (!fired && !done.empty() && m - nseen <= kTail && nseen < m) {
                     fired = true;
-                    const int st = early(user, (int)done.size(), done.data());
-                    if (st) first_err = st;
+                    first_err = early(user, (int)done.size(), done.data());
                 }
                 if (nseen == m) break;
                 if (ended) {   // the kernel ended without every record: a device error
@@ -2407,23 +2153,31 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
                 }
                 std::this_thread::yield();
             }
-            cudaError_t e = ibip_sync(ctx, s);
+        } else {
+            // steps and status of every image
+            int64_t *ho = (int64_t *)ctx->h_pinned;
+            cudaMemcpy2DAsync(ho, 2 * sizeof(int64_t), outs, kOut, 2 * sizeof(int64_t), m, cudaMemcpyDeviceToHost, s);
+            const cudaError_t e = ibip_sync(ctx, s);
             if (e != cudaSuccess) return ibip_cuda_status(e);
-            return first_err;
-        }
-        // steps and status of every job
-        int64_t *ho = (int64_t *)ctx->h_pinned;
-        for (int q = 0; q < m; q++) cudaMemcpyAsync(ho + 2 * q, outs[idx[q]], 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-        cudaError_t e = ibip_sync(ctx, s);
-        if (e != cudaSuccess) return ibip_cuda_status(e);
-        for (int q = 0; q < m; q++) {
-            it[idx[q]].n_steps = ho[2 * q];
-            it[idx[q]].status = (int)ho[2 * q + 1];
+            for (int q = 0; q < m; q++) {
+                if (ho[2 * q + 1] == kFloodGiveUp) { single.push_back(idx[q]); continue; }
+                it[idx[q]].n_steps = ho[2 * q];
+                it[idx[q]].status = (int)ho[2 * q + 1];
+            }
         }
     } else {
         ibip_prof_end(ctx, IBIP_K_RANK);
-        cudaError_t e = ibip_sync(ctx, s);
-        if (e != cudaSuccess) return ibip_cuda_status(e);
     }
-    return IBIP_OK;
+    const cudaError_t e = ibip_sync(ctx, s);
+    if (e != cudaSuccess) return ibip_cuda_status(e);
+    for (int j : single) {
+        int64_t out[kNOut] = {0};
+        ibip_prof_begin(ctx, IBIP_K_RANK);
+        const int st = loop_run(ctx, it[j].dt2, it[j].d, it[j].inlet, it[j].max_steps, it[j].seq, it[j].step_r2,
+                                it[j].step_centre, it[j].cap, maxd[j], npore[j], hasinf[j], nullptr, 0, 0, out);
+        if (st) return st;
+        it[j].n_steps = out[0];
+        it[j].status = (int)out[1];
+    }
+    return first_err;
 }
