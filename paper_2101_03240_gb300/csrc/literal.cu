@@ -393,6 +393,396 @@ __global__ void k_lit_bval(const int32_t *incl, int maxd, int B, int hasinf, int
         if (incl[v] != incl[v - 1]) bval[B - incl[v]] = v;
 }
 
+// ------------------------------------------------------- walk, then stamp --
+// The one-image schedule.  Which voxels become insertion points, and when,
+// does not depend on the spheres: it is a flood of the voxel graph, all
+// pending voxels of the largest value at a time.  So one CTA walks the flood
+// and writes only cstep, and one wide launch stamps all spheres afterwards,
+// seq[p] = the smallest cstep among the centres whose sphere holds p.  Walked
+// together with the stamping on a cluster a step cost ~5 us (two cluster
+// barriers, remote counters, the spheres' memory traffic).  Values up to
+// kWalkVals (bookkeeping by value in shared memory); larger ones take the
+// cluster kernel.
+constexpr int kWT = 512;            // threads of the walk
+constexpr int kWalkVals = 4095;     // largest squared distance it takes
+constexpr int kSoloPts = 21;        // points of a step run on one warp (four passes of 32 lanes)
+constexpr int kCtaPts = 512;        // points of a step run on one CTA
+constexpr int kWalkRing = 16;       // last entries of each list kept in shared memory (fewer for large values)
+
+// The state and step images of the walk have a border of one solid voxel, so
+// that a neighbour is an offset and no step needs coordinates: voxel
+// (x, y, z) is ((x + 1) * (ny + 2) + y + 1) * (nz + 2) + z + 1.
+struct Walk {
+    int nx, ny, nz, inlet, maxd, npore, ring;   // ring: entries per list in shared memory, a power of two
+    const int32_t *dt2;
+    int32_t *seq, *cstep, *step_r2, *step_count;
+    int64_t cap, max_steps;
+    unsigned short *state;   // value; bit 15: queued (zero at the border, cleared before)
+    int32_t *when;           // step of each insertion point, 0 before (cleared before)
+    int32_t *list;           // queued voxels of value v: entries start[v] .. start[v] + cnt[v]
+    int32_t *cnt, *start;    // [maxd + 1]
+    int64_t *out;
+};
+
+// state, sequence (-1 on pore) and the number of voxels of each value; a warp
+// per row
+__global__ void k_walk_init(Walk a)
+{
+    extern __shared__ int32_t s_cnt[];
+    for (int i = threadIdx.x; i <= a.maxd; i += blockDim.x) s_cnt[i] = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5, rows = a.nx * a.ny;
+    for (int r = blockIdx.x * wpb + (threadIdx.x >> 5); r < rows; r += gridDim.x * wpb) {
+        const int x = r / a.ny, y = r - x * a.ny;
+        const int64_t vb = (int64_t)r * a.nz;
+        unsigned short *sp = a.state + ((int64_t)(x + 1) * (a.ny + 2) + y + 1) * (a.nz + 2) + 1;
+        for (int z = lane; z < a.nz; z += 32) {
+            const int d = max(a.dt2[vb + z], 0);
+            a.seq[vb + z] = d > 0 ? -1 : 0;
+            sp[z] = (unsigned short)d;
+            if (d > 0) atomicAdd(s_cnt + d, 1);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i <= a.maxd; i += blockDim.x)
+        if (s_cnt[i]) atomicAdd(a.cnt + i, s_cnt[i]);
+}
+
+// start = exclusive prefix of cnt, cnt = 0 (one block)
+__global__ void __launch_bounds__(1024) k_walk_start(Walk a)
+{
+    __shared__ int s_w[32];
+    __shared__ int s_run;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_run = 0;
+    __syncthreads();
+    for (int i0 = 0; i0 <= a.maxd; i0 += 1024) {
+        const int i = i0 + threadIdx.x, n = i <= a.maxd ? a.cnt[i] : 0;
+        int inc = n;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        if (lane == 31) s_w[w] = inc;
+        __syncthreads();
+        int base = s_run, all = 0;
+        for (int q = 0; q < 32; q++) {
+            if (q < w) base += s_w[q];
+            all += s_w[q];
+        }
+        if (i <= a.maxd) {
+            a.start[i] = base + inc - n;
+            a.cnt[i] = 0;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) s_run += all;
+        __syncthreads();
+    }
+}
+
+// The first candidates, the inlet face and its face neighbours: the two
+// layers of voxels at the face.
+__global__ void k_walk_seed(Walk a)
+{
+    const int ax = a.inlet >> 1, len = ax == 0 ? a.nx : ax == 1 ? a.ny : a.nz;
+    const int n0 = ax == 0 ? a.ny : a.nx, n1 = ax == 2 ? a.ny : a.nz;
+    const int64_t nf = (int64_t)n0 * n1, n = nf * min(2, len);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int layer = (int)(i / nf), p = (int)((i - layer * nf) / n1), q = (int)((i - layer * nf) % n1);
+        const int fixed = (a.inlet & 1) ? len - 1 - layer : layer;
+        const int py = a.ny + 2, pz = a.nz + 2;
+        const int64_t v = ax == 0 ? d_lin(fixed + 1, p + 1, q + 1, py, pz)
+                          : ax == 1 ? d_lin(p + 1, fixed + 1, q + 1, py, pz) : d_lin(p + 1, q + 1, fixed + 1, py, pz);
+        const int s = a.state[v];
+        if (!s) continue;
+        a.state[v] = (unsigned short)(s | 0x8000);
+        const unsigned act = __activemask(), peers = __match_any_sync(act, s);
+        const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
+        int pos = 0;
+        if (lane == leader) pos = atomicAdd(a.cnt + s, __popc(peers));
+        pos = __shfl_sync(peers, pos, leader) + __popc(peers & ((1u << lane) - 1));
+        a.list[a.start[s] + pos] = (int32_t)v;
+    }
+}
+
+// The flood, on one cluster.  CTA 0 owns the bookkeeping.  Steps of up to
+// kSoloPts points run on its warp 0 alone: only this SM touches the state
+// image then, so its loads hit L1 and a step costs a few hundred cycles;
+// voxels met by several lanes are queued by the lowest.  Steps of up to
+// kCtaPts points run on CTA 0, larger ones on every CTA (a value is 1 or 2
+// for most points of a pack, a few steps of 10^5 points each), the others
+// waiting at the cluster barrier in between; both queue through an atomic OR
+// on the state word.
+__global__ void __launch_bounds__(kWT, 1) k_walk(Walk a)
+{
+    extern __shared__ int32_t s_walk[];
+    __shared__ int s_t, s_h, s_n, s_stop, s_k;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), ncta = (int)cl.num_blocks();
+    const int nv = a.maxd + 1, nw = (nv + 31) >> 5;
+    int32_t *const tail = s_walk, *const head = tail + nv, *const start = head + nv, *const rr = start + nv;
+    uint32_t *const ne = (uint32_t *)(rr + nv);
+    int32_t *const ring = (int32_t *)(ne + nw);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const uint32_t rm = (uint32_t)a.ring - 1;
+    for (int i = tid; i < nw; i += kWT) ne[i] = 0u;
+    __syncthreads();
+    for (int i = tid; i < nv; i += kWT) {
+        const int n = a.cnt[i];
+        tail[i] = n;
+        head[i] = 0;
+        start[i] = a.start[i];
+        const int R = d_isqrt(i);   // trunc(dt)
+        rr[i] = R * R;
+        if (n && i) atomicOr(ne + (i >> 5), 1u << (i & 31));
+        for (int p = max(0, n - a.ring); p < n; p++) ring[i * a.ring + (p & rm)] = a.list[a.start[i] + p];
+    }
+    __syncthreads();
+    const int rsz = a.ring, oy = a.nz + 2, ox = (a.ny + 2) * oy;
+    unsigned short *const state = a.state;
+    int32_t *const list = a.list, *const when = a.when;
+    // offset of neighbour dir
+    auto offset = [&](int dir) {
+        const int o = dir < 2 ? ox : dir < 4 ? oy : 1;
+        return (dir & 1) ? o : -o;
+    };
+    const int q0 = lane / 6, off0 = offset(lane - 6 * q0);   // first pass: point and offset of this lane
+    // A step of n points on the CTAs first .. first + count - 1 of the
+    // cluster: points and neighbours dealt to all threads, the bookkeeping in
+    // CTA 0's shared memory, one counter update per value and warp.
+    auto wide_step = [&](int32_t *tail0, uint32_t *ne0, int32_t *ring0, int t, int h, int n, int k, int part, int parts) {
+        const int32_t *pts = list + start[t] + h;
+        const int64_t all = (int64_t)n * 6, stride = (int64_t)parts * kWT;
+        for (int64_t i0 = (int64_t)part * kWT + (tid & ~31); i0 < all; i0 += 2 * stride) {
+            int v[2], val[2];
+#pragma unroll
+            for (int j = 0; j < 2; j++) {
+                const int64_t i = i0 + j * stride + lane;
+                v[j] = -1;
+                if (i >= all) continue;
+                const int q = (int)(i / 6), dir = (int)(i - (int64_t)q * 6);
+                const int u = __ldcg(pts + q);
+                if (dir == 0) when[u] = k;
+                v[j] = u + offset(dir);
+            }
+            // a look first: most neighbours are solid or queued already
+#pragma unroll
+            for (int j = 0; j < 2; j++) val[j] = v[j] >= 0 ? (int)__ldcg(state + v[j]) : 0;
+#pragma unroll
+            for (int j = 0; j < 2; j++) {
+                if (val[j] == 0 || (val[j] & 0x8000)) { val[j] = 0; continue; }
+                const uint32_t bit = (v[j] & 1) ? 0x80000000u : 0x8000u;
+                if (atomicOr((uint32_t *)state + (v[j] >> 1), bit) & bit) val[j] = 0;
+            }
+#pragma unroll
+            for (int j = 0; j < 2; j++) {
+                const unsigned peers = __match_any_sync(0xffffffffu, val[j]);
+                const int leader = __ffs(peers) - 1;
+                int pos = 0;
+                if (val[j] && lane == leader) {
+                    pos = atomicAdd(tail0 + val[j], __popc(peers));
+                    atomicOr(ne0 + (val[j] >> 5), 1u << (val[j] & 31));
+                }
+                pos = __shfl_sync(0xffffffffu, pos, leader) + __popc(peers & ((1u << lane) - 1));
+                if (!val[j]) continue;
+                list[start[val[j]] + pos] = v[j];
+                ring0[val[j] * rsz + (pos & rm)] = v[j];
+            }
+        }
+    };
+    if (rank == 0) {
+        int64_t k = 0;   // steps (warp 0)
+        const int64_t cap = a.cap, last = min(a.max_steps, (int64_t)a.npore);   // every step consumes a voxel
+        int32_t *const step_r2 = a.step_r2, *const step_count = a.step_count;
+        for (;;) {
+            if (tid < 32) {
+                int stop = 0, t = 0, h = 0, n = 0;
+                for (;;) {
+                    // the largest value with pending voxels
+                    if (nw <= 32) {
+                        const uint32_t m = lane < nw ? *(volatile uint32_t *)(ne + nw - 1 - lane) : 0u;
+                        const unsigned bal = __ballot_sync(0xffffffffu, m != 0u);
+                        const int l = __ffs(bal) - 1;
+                        t = ((nw - 1 - l) << 5) + 31 - __clz(__shfl_sync(0xffffffffu, m, l & 31));
+                        if (!bal) t = -1;
+                    } else {
+                        t = -1;
+                        for (int w0 = nw - 1; w0 >= 0 && t < 0; w0 -= 32) {
+                            const int w = w0 - lane;
+                            const uint32_t m = w >= 0 ? *(volatile uint32_t *)(ne + w) : 0u;
+                            const unsigned bal = __ballot_sync(0xffffffffu, m != 0u);
+                            if (bal) {
+                                const int l = __ffs(bal) - 1;
+                                t = ((w0 - l) << 5) + 31 - __clz(__shfl_sync(0xffffffffu, m, l));
+                            }
+                        }
+                    }
+                    if (t < 0) { stop = 1; break; }
+                    if (k >= last) { stop = k >= a.max_steps ? 2 : 3; break; }
+                    h = *(volatile int32_t *)(head + t);
+                    const int e = *(volatile int32_t *)(tail + t);
+                    const uint32_t nt = *(volatile uint32_t *)(ne + (t >> 5));
+                    n = e - h;
+                    k++;
+                    __syncwarp();
+                    // (every lane writes the same, without a branch)
+                    *(volatile int32_t *)(head + t) = e;
+                    *(volatile uint32_t *)(ne + (t >> 5)) = nt & ~(1u << (t & 31));   // empty until this step queues into it
+                    if (n > kSoloPts) break;
+                    if (k <= cap) {
+                        step_r2[k - 1] = rr[t];
+                        step_count[k - 1] = n;
+                    }
+                    // queue what is pore, new and not met by a lower lane
+                    auto meet = [&](int v) {
+                        const int val = v >= 0 ? (int)state[v] : 0;
+                        const bool fresh = (unsigned)(val - 1) < 0x7fffu;
+                        const unsigned some = __ballot_sync(0xffffffffu, fresh);
+                        if (!some) return;
+                        bool first = fresh;
+                        if (n > 1) {
+                            const unsigned same = __match_any_sync(0xffffffffu, fresh ? v : -1 - lane);
+                            first = fresh && lane == __ffs(same) - 1;
+                        }
+                        if (first) {
+                            const int pos = atomicAdd(tail + val, 1), base = start[val];
+                            state[v] = (unsigned short)(val | 0x8000);
+                            atomicOr(ne + (val >> 5), 1u << (val & 31));
+                            ring[val * rsz + (pos & rm)] = v;
+                            list[base + pos] = v;
+                            // its own neighbours' rows, for the step that takes it
+                            asm volatile("prefetch.global.L1 [%0];" ::"l"(state + v - oy));
+                            asm volatile("prefetch.global.L1 [%0];" ::"l"(state + v + oy));
+                            asm volatile("prefetch.global.L1 [%0];" ::"l"(state + v - ox));
+                            asm volatile("prefetch.global.L1 [%0];" ::"l"(state + v + ox));
+                        }
+                        __syncwarp();
+                    };
+                    if (n <= 5 && n <= rsz) {   // one pass, the points from the ring
+                        int v = -1;
+                        if (q0 < n) {
+                            const int u = ring[t * rsz + ((h + q0) & rm)];
+                            if (lane == 6 * q0) when[u] = (int32_t)k;
+                            v = u + off0;
+                        }
+                        __syncwarp();
+                        meet(v);
+                    } else {
+                        // the points of all passes first, since pushes reuse the ring
+                        int v[4];
+#pragma unroll
+                        for (int j = 0; j < 4; j++) {
+                            const int i = lane + 32 * j, q = i / 6, dir = i - 6 * q, p = h + q;
+                            v[j] = -1;
+                            if (q >= n) continue;
+                            const int u = e - p <= rsz ? ring[t * rsz + (p & rm)] : __ldcg(list + start[t] + p);
+                            if (dir == 0) when[u] = (int32_t)k;
+                            v[j] = u + offset(dir);
+                        }
+                        __syncwarp();
+#pragma unroll
+                        for (int j = 0; j < 4; j++)
+                            if (32 * j < 6 * n) meet(v[j]);
+                    }
+                }
+                if (lane == 0) {
+                    s_stop = stop; s_t = t; s_h = h; s_n = n; s_k = (int)k;
+                    if (!stop && k <= a.cap) {
+                        a.step_r2[k - 1] = rr[t];
+                        a.step_count[k - 1] = n;
+                    }
+                }
+            }
+            __syncthreads();
+            const bool wide = s_n > kCtaPts && ncta > 1;
+            if (s_stop) break;
+            if (wide) cl.sync();
+            wide_step(tail, ne, ring, s_t, s_h, s_n, s_k, 0, wide ? ncta : 1);
+            if (wide) cl.sync();
+            else __syncthreads();
+        }
+        if (tid == 0) {
+            a.out[0] = k;
+            a.out[1] = s_stop == 2 ? IBIP_ERR_STEP_LIMIT : (s_stop == 3 ? IBIP_ERR_BOUNDS : IBIP_OK);
+        }
+        cl.sync();   // the others read s_stop
+    } else {
+        const int *const r_t = cl.map_shared_rank(&s_t, 0), *const r_h = cl.map_shared_rank(&s_h, 0);
+        const int *const r_n = cl.map_shared_rank(&s_n, 0), *const r_k = cl.map_shared_rank(&s_k, 0);
+        const int *const r_stop = cl.map_shared_rank(&s_stop, 0);
+        int32_t *const tail0 = cl.map_shared_rank(tail, 0), *const ring0 = cl.map_shared_rank(ring, 0);
+        uint32_t *const ne0 = cl.map_shared_rank(ne, 0);
+        for (;;) {
+            cl.sync();
+            if (*(volatile const int *)r_stop) break;
+            wide_step(tail0, ne0, ring0, *(volatile const int *)r_t, *(volatile const int *)r_h,
+                      *(volatile const int *)r_n, *(volatile const int *)r_k, rank, ncta);
+            cl.sync();
+        }
+    }
+    cl.sync();   // CTA 0's shared memory is still read above
+}
+
+// All spheres: seq[p] = min cstep over the centres within floor(sqrt(dt2)) of
+// p (as unsigned, so that -1 is the largest).  A centre whose face neighbour
+// has a radius larger by one and no later step is skipped: its sphere lies
+// inside the neighbour's.  A warp takes 32 voxels; spheres of radius 1 are
+// written by their lane, the others by the whole warp.
+__global__ void __launch_bounds__(256) k_walk_stamp(Walk a)
+{
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    const int segs = (a.nz + 31) >> 5;   // a warp takes 32 voxels of a row
+    const int64_t nyz = (int64_t)a.ny * a.nz, units = (int64_t)a.nx * a.ny * segs;
+    const int oy = a.nz + 2, ox = (a.ny + 2) * oy;
+    uint32_t *seq = (uint32_t *)a.seq;
+    for (int64_t un = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); un < units; un += (int64_t)gridDim.x * wpb) {
+        const int row = (int)(un / segs), x = row / a.ny, y = row - x * a.ny;
+        const int z = (int)(un - (int64_t)row * segs) * 32 + lane;
+        const int64_t v = (int64_t)row * a.nz + z;
+        const int64_t u = ((int64_t)(x + 1) * (a.ny + 2) + y + 1) * oy + z + 1;
+        int k = 0, R = 0;
+        if (z < a.nz) {
+            k = a.when[u];
+            a.cstep[v] = k;
+        }
+        bool on = k > 0;
+        if (on) {
+            R = d_isqrt(a.dt2[v]);
+            const int big = (R + 1) * (R + 1);
+            // a neighbour's value and step (solid and border voxels: step 0)
+            auto holds = [&](int64_t o) {
+                const int kn = a.when[u + o];
+                return kn > 0 && kn <= k && (int)(a.state[u + o] & 0x7fff) >= big;
+            };
+            if (holds(-1) || holds(1) || holds(-oy) || holds(oy) || holds(-ox) || holds(ox)) on = false;
+        }
+        if (on && R == 1) {
+            atomicMin(seq + v, (uint32_t)k);
+            if (z > 0) atomicMin(seq + v - 1, (uint32_t)k);
+            if (z < a.nz - 1) atomicMin(seq + v + 1, (uint32_t)k);
+            if (y > 0) atomicMin(seq + v - a.nz, (uint32_t)k);
+            if (y < a.ny - 1) atomicMin(seq + v + a.nz, (uint32_t)k);
+            if (x > 0) atomicMin(seq + v - nyz, (uint32_t)k);
+            if (x < a.nx - 1) atomicMin(seq + v + nyz, (uint32_t)k);
+        }
+        for (unsigned m = __ballot_sync(0xffffffffu, on && R > 1); m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const int cz = __shfl_sync(0xffffffffu, z, src), r = __shfl_sync(0xffffffffu, R, src);
+            const uint32_t lab = (uint32_t)__shfl_sync(0xffffffffu, k, src);
+            const int side = 2 * r + 1;
+            for (int q = lane; q < side * side; q += 32) {
+                const int dx = q / side - r, dy = q % side - r, e = r * r - dx * dx - dy * dy;
+                const int X = x + dx, Y = y + dy;
+                if (e < 0 || X < 0 || Y < 0 || X >= a.nx || Y >= a.ny) continue;
+                const int h = d_isqrt(e);
+                const int z0 = max(cz - h, 0), z1 = min(cz + h, a.nz - 1);
+                uint32_t *p = seq + ((int64_t)X * a.ny + Y) * a.nz;
+                for (int zz = z0; zz <= z1; zz++) atomicMin(p + zz, lab);
+            }
+        }
+    }
+}
+
 }  // namespace
 
 // Largest cluster (16, 8, 4 or 2 CTAs of 1024 threads with `book` bytes of
@@ -420,6 +810,82 @@ static int lit_cluster_size(size_t book)
     return 0;
 }
 
+// The walk schedule (k_walk) for values up to kWalkVals.
+static int walk_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps, int32_t *seq,
+                    int32_t *cstep, int32_t *step_r2, int32_t *step_count, int64_t cap, int maxd, int npore,
+                    int64_t *h_out)
+{
+    cudaStream_t s = ctx->stream;
+    const int nv = maxd + 1;
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const int64_t Np = (int64_t)(d.nx + 2) * (d.ny + 2) * (d.nz + 2);
+    const size_t o_state = up((size_t)npore * 4), o_when = o_state + up((size_t)Np * 2 + 16),
+                 o_cnt = o_when + up((size_t)Np * 4), o_start = o_cnt + up((size_t)nv * 4), o_out = o_start + up((size_t)nv * 4), total = o_out + up(64);
+    char *w = (char *)ibip_scratch(ctx, SC_LIT, total);
+    if (!w) return IBIP_ERR_OOM;
+    Walk a;
+    a.nx = d.nx; a.ny = d.ny; a.nz = d.nz; a.inlet = inlet; a.maxd = maxd; a.npore = npore;
+    a.dt2 = dt2; a.seq = seq; a.cstep = cstep; a.step_r2 = step_r2; a.step_count = step_count;
+    a.cap = cap; a.max_steps = max_steps;
+    a.list = (int32_t *)w;
+    a.state = (unsigned short *)(w + o_state);
+    a.when = (int32_t *)(w + o_when);
+    a.cnt = (int32_t *)(w + o_cnt);
+    a.start = (int32_t *)(w + o_start);
+    a.out = (int64_t *)(w + o_out);
+    a.ring = kWalkRing;
+    while (a.ring > 1 && (size_t)nv * a.ring * 4 > 96 * 1024) a.ring /= 2;
+    cudaMemsetAsync(w + o_state, 0, o_start - o_state, s);   // state, when, cnt
+    const int gs = ctx->sm_count * 8;
+    k_walk_init<<<gs, 256, (size_t)nv * 4, s>>>(a);
+    IBIP_LAUNCH(ctx);
+    k_walk_start<<<1, 1024, 0, s>>>(a);
+    IBIP_LAUNCH(ctx);
+    const int ax = inlet >> 1;
+    const int64_t nf = 2 * (ax == 0 ? (int64_t)d.ny * d.nz : ax == 1 ? (int64_t)d.nx * d.nz : (int64_t)d.nx * d.ny);
+    k_walk_seed<<<(int)std::max<int64_t>(1, std::min<int64_t>(gs, (nf + 255) / 256)), 256, 0, s>>>(a);
+    IBIP_LAUNCH(ctx);
+    ibip_prof_end(ctx, IBIP_K_RANK);
+    ibip_prof_begin(ctx, IBIP_K_INVADE);
+    const size_t book = ((size_t)nv * (4 + a.ring) + (nv + 31) / 32) * 4;
+    cudaFuncSetAttribute(k_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLitSmem);
+    cudaFuncSetAttribute(k_walk, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int cs = 16; cs >= 1; cs /= 2) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = cs;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(cs);
+        cfg.blockDim = dim3(kWT);
+        cfg.dynamicSmemBytes = book;
+        cfg.stream = s;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, k_walk, &cfg) != cudaSuccess || fit < 1) {
+            cudaGetLastError();
+            if (cs == 1) return IBIP_ERR_CUDA;
+            continue;
+        }
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_walk, a);
+        if (e != cudaSuccess) return ibip_cuda_status(e);
+        break;
+    }
+    IBIP_LAUNCH(ctx);
+    k_walk_stamp<<<(int)std::max<int64_t>(1, std::min<int64_t>(gs, (nvox(d) + 255) / 256)), 256, 0, s>>>(a);
+    IBIP_LAUNCH(ctx);
+    ibip_prof_end(ctx, IBIP_K_INVADE);
+    int64_t *ho = (int64_t *)ctx->h_pinned;
+    cudaMemcpyAsync(ho, a.out, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    const cudaError_t e = ibip_sync(ctx, s);
+    if (e != cudaSuccess) return ibip_cuda_status(e);
+    h_out[0] = ho[0];
+    h_out[1] = ho[1];
+    return IBIP_OK;
+}
+
 int ibip_literal_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps, int32_t *seq,
                      int32_t *cstep, int32_t *step_r2, int32_t *step_count, int64_t cap, int64_t *h_out)
 {
@@ -436,6 +902,9 @@ int ibip_literal_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, 
     cudaMemcpyAsync(h, stats, 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
     if (ibip_sync(ctx, s) != cudaSuccess) return IBIP_ERR_CUDA;
     const int maxd = h[0], npore = h[1], hasinf = h[2];
+    if (!hasinf && npore > 0 && maxd <= kWalkVals &&
+        (int64_t)(d.nx + 2) * (d.ny + 2) * (d.nz + 2) < (1ll << 31))
+        return walk_run(ctx, dt2, d, inlet, max_steps, seq, cstep, step_r2, step_count, cap, maxd, npore, h_out);
     k_lit_init<<<gs, 256, 0, s>>>(dt2, N, seq, cstep);
     IBIP_LAUNCH(ctx);
     if (npore == 0) {
