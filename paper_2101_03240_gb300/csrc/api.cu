@@ -35,7 +35,6 @@ int ibip_level_counts(ibip_ctx *ctx, const int32_t *level, ibip_dims d, int L, i
 namespace {
 
 constexpr int kMaxDim = 16384;
-constexpr int kMaxRounds = 1 << 20;
 
 bool dims_ok(ibip_dims d)
 {
@@ -180,7 +179,7 @@ int ibip_run_job(ibip_ctx *ctx, ibip_job &J)
     if (J.trapped) {
         int32_t *M = (int32_t *)ibip_scratch(ctx, SC_MM, (size_t)nvox(J.dims) * sizeof(int32_t));
         if (!M) return IBIP_ERR_OOM;
-        st = ibip_maximin_launch(ctx, J.seq, J.dims, J.outlet, M, kMaxRounds);
+        st = ibip_maximin_launch(ctx, J.seq, J.dims, J.outlet, M);
         if (!st) st = ibip_trap_finish(ctx, J.seq, M, J.dims, 0, J.trapped, J.seq_out);
         if (st) return st;
         if (J.seq_out) curve_seq = J.seq_out;
@@ -206,7 +205,7 @@ struct BatchPost {
     int early_err = IBIP_OK;
 };
 
-int batch_post_group(BatchPost &P, const std::vector<int> &group, bool shared_device)
+int batch_post_group(BatchPost &P, const std::vector<int> &group)
 {
     ibip_ctx *ctx = P.ctx;
     std::vector<IbipMaximinJob> mj;
@@ -220,16 +219,7 @@ int batch_post_group(BatchPost &P, const std::vector<int> &group, bool shared_de
         mj.push_back(IbipMaximinJob{J.seq, J.dims, J.outlet, P.M + P.M_off[j]});
         mj_of.push_back(j);
     }
-    // Beside the batch's last running invasion CTAs no cooperative grid may
-    // start.  Several images run on the widest path's work queue, whose
-    // blocks take the free SMs without needing all to be resident (the
-    // remaining invasion CTAs are resident already, so nothing waits for
-    // those SMs); a single image, which could get the cooperative rounds,
-    // runs one launch per round instead.
-    const int keep_nc = ctx->no_coop;
-    ctx->no_coop = shared_device && mj.size() == 1 ? 1 : keep_nc;
-    int st = mj.empty() ? IBIP_OK : ibip_maximin_multi(ctx, (int)mj.size(), mj.data(), kMaxRounds);
-    ctx->no_coop = keep_nc;
+    const int st = mj.empty() ? IBIP_OK : ibip_maximin_multi(ctx, (int)mj.size(), mj.data());
     if (st) {
         if (st != IBIP_ERR_NOT_CONVERGED) return st;
         for (int j : mj_of) P.jobs[j].status = st;
@@ -258,7 +248,7 @@ int batch_early(void *user, int n_done, const int *done)
     for (int j : group) P.early[j] = 1;
     cudaStream_t keep = ctx->stream;
     ctx->stream = ctx->stream2;
-    const int st = batch_post_group(P, group, true);
+    const int st = batch_post_group(P, group);
     ctx->stream = keep;
     P.early_err = st;
     return st;
@@ -640,7 +630,7 @@ int ibip_trapping(ibip_ctx *ctx, const int32_t *seq, ibip_dims dims, int outlet,
     DeviceGuard g(ctx->device);
     int32_t *M = (int32_t *)ibip_scratch(ctx, SC_MM, (size_t)nvox(dims) * sizeof(int32_t));
     if (!M) return IBIP_ERR_OOM;
-    int st = ibip_maximin_launch(ctx, seq, dims, outlet, M, kMaxRounds);
+    int st = ibip_maximin_launch(ctx, seq, dims, outlet, M);
     if (st) return st;
     st = ibip_trap_finish(ctx, seq, M, dims, rerank, trapped, seq_out);
     if (st) return st;
@@ -658,7 +648,7 @@ int ibip_trapping_ex(ibip_ctx *ctx, const int32_t *seq, ibip_dims dims, int outl
     DeviceGuard g(ctx->device);
     int32_t *M = (int32_t *)ibip_scratch(ctx, SC_MM, (size_t)nvox(dims) * sizeof(int32_t));
     if (!M) return IBIP_ERR_OOM;
-    int st = ibip_maximin_launch(ctx, seq, dims, outlet, M, kMaxRounds);
+    int st = ibip_maximin_launch(ctx, seq, dims, outlet, M);
     if (st) return st;
     st = ibip_trap_finish(ctx, seq, M, dims, 1, trapped, seq_out, step_r2, n_steps, step_r2_out, h_n_steps_out);
     if (st) return st;
@@ -695,7 +685,7 @@ int ibip_morph_drainage_ex(ibip_ctx *ctx, const uint8_t *image, const int32_t *d
     int st = ibip_level_init(ctx, image, dims, level);
     if (st) return st;
     if (n_levels == 0) return ibip_cuda_status(ibip_sync(ctx, ctx->stream));
-    st = ibip_maximin_launch(ctx, dt2, dims, inlet, W, kMaxRounds);
+    st = ibip_maximin_launch(ctx, dt2, dims, inlet, W);
     if (st) return st;
     // radii above the largest widest-path value trim to the empty set: skip
     int wmax = 0;
@@ -773,19 +763,23 @@ int ibip_invade_batched(ibip_ctx *ctx, int32_t n, ibip_job *jobs)
     P.it = it.data();
     P.M_off.assign(n, -1);
     P.early.assign(n, 0);
-    int64_t mm_total = 0, nt_total = 0, cnt_total = 0;
+    int64_t mm_total = 0, cnt_total = 0;
     for (int j = 0; j < n; j++) {
         const ibip_job &J = jobs[j];
         if (J.trapped) {
             P.M_off[j] = mm_total;
             mm_total += (nvox(J.dims) + 63) & ~(int64_t)63;
-            nt_total += (int64_t)((J.dims.nx + 3) / 4) * ((J.dims.ny + 7) / 8) * ((J.dims.nz + 31) / 32);
         }
         if (J.sat_per_step) cnt_total += nvox(J.dims) + 2;
     }
     P.M = mm_total ? (int32_t *)ibip_scratch(ctx, SC_MM, (size_t)mm_total * sizeof(int32_t)) : nullptr;
-    const size_t tile_bytes = ((size_t)n * 64 + 255) / 256 * 256 + ((size_t)3 * nt_total + 2 * ((1 << 16) + 2) + 4) * 4;
-    if ((mm_total && !P.M) || (nt_total && !ibip_scratch(ctx, SC_TILE, tile_bytes)) ||
+    // the widest path's tables: basins are a few percent of the voxels
+    const size_t basins = (size_t)mm_total / 8 + 1024;
+    if ((mm_total && (!P.M || !ibip_scratch(ctx, SC_TILE, (size_t)n * 128 + 1024) ||
+                      !ibip_scratch(ctx, SC_OKEY, basins * 8) || !ibip_scratch(ctx, SC_HIST, basins * 8) ||
+                      !ibip_scratch(ctx, SC_RANK, (size_t)mm_total * 4) ||
+                      !ibip_scratch(ctx, SC_G2, (size_t)mm_total * 4) ||
+                      !ibip_scratch(ctx, SC_LIST, (size_t)mm_total * 4))) ||
         !ibip_scratch(ctx, SC_HIST, ibip_curve_batch_bytes(n, cnt_total)) ||
         !ibip_scratch(ctx, SC_SCAN, ibip_scan_scratch_bytes(cnt_total + 1)) || !ibip_scratch(ctx, SC_SMALL, kSmallBytes))
         return IBIP_ERR_OOM;
@@ -796,7 +790,7 @@ int ibip_invade_batched(ibip_ctx *ctx, int32_t n, ibip_job *jobs)
     std::vector<int> rest;
     for (int j = 0; j < n; j++)
         if (!P.early[j]) rest.push_back(j);
-    st = batch_post_group(P, rest, false);
+    st = batch_post_group(P, rest);
     if (st) return st;
     cudaError_t e = ibip_sync(ctx, s);
     if (e != cudaSuccess) return ibip_cuda_status(e);

@@ -23,7 +23,7 @@ enum ScratchSlot {
     SC_MAT,       // int32 per-(bucket, chunk) counts
     SC_SCAN,      // scan partial sums
     SC_MM,        // int32[N]      maximin field
-    SC_TILE,      // u8 tile activity flags
+    SC_TILE,      // widest path: job table, counters
     SC_HIST,      // int32 histogram
     SC_SMALL,     // small device scalars
     SC_LIST,      // int32 overflow work lists of the invasion kernel
@@ -63,7 +63,8 @@ struct ibip_ctx {
     // arena_size) and never freed; a request that does not fit fails.
     char *arena;
     size_t arena_size, arena_used;
-    // Kernels share the device with other streams: no cooperative launches.
+    // Kernels share the device with other streams: no cooperative launches
+    // (the invasion runs on one cluster).
     int no_coop;
     // Server slots: the invasion kernel goes to this stream (of the
     // device's highest priority, owned by the context, with an event that
@@ -169,16 +170,15 @@ int ibip_dilate_first_level_launch(ibip_ctx *ctx, const uint8_t *fl, int32_t T, 
 int ibip_max_launch(ibip_ctx *ctx, const int32_t *a, int64_t n, int *h_max);
 // Maximin propagation from a face through voxels with val != 0 (val == -1
 // counts as +inf).  Writes M (-1 where unreachable).
-int ibip_maximin_launch(ibip_ctx *ctx, const int32_t *val, ibip_dims d, int face, int32_t *M,
-                        int max_rounds);
-// The same for several images in one cooperative launch.
+int ibip_maximin_launch(ibip_ctx *ctx, const int32_t *val, ibip_dims d, int face, int32_t *M);
+// The same for several images at once.
 struct IbipMaximinJob {
     const int32_t *val;
     ibip_dims d;
     int face;
     int32_t *M;
 };
-int ibip_maximin_multi(ibip_ctx *ctx, int n, const IbipMaximinJob *jobs, int max_rounds);
+int ibip_maximin_multi(ibip_ctx *ctx, int n, const IbipMaximinJob *jobs);
 // Pore statistics of a dt2 image: stats[0] = largest finite value, [1] =
 // pore voxels, [2] = 1 if any value is infinite (stats zeroed by the caller).
 int ibip_stats_launch(ibip_ctx *ctx, const int32_t *dt2, int64_t N, int *stats);

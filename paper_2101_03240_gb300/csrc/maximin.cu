@@ -1,755 +1,527 @@
-// maximin.cu -- widest-path (maximin) propagation from an image face, used
-// by defending-phase trapping (Section 2.2.3) and by the trimming step of
+// maximin.cu -- widest-path (maximin) values from an image face, used by
+// defending-phase trapping (Section 2.2.3) and by the trimming step of
 // morphological-opening drainage (Section 2.4.1).
 //
 // For a value field val (0 = blocked, -1 = +infinity, else the value) and a
 // face F, M[v] is the largest, over 6-paths through unblocked voxels from a
 // voxel of F to v, of the smallest value on the path (v included); -1 where
-// no such path exists.  M is the least fixed point of
-//     M[v] = max(M[v], min(val[v], max over neighbours u of M[u]))
-// started from M = val on F.  Trapping thresholds it against seq (a voxel of
-// step k is trapped iff M < k); opening keeps {M >= T}.
+// no such path exists.  Trapping thresholds it against seq (a voxel of step
+// k is trapped iff M < k); opening keeps {M >= T}.
 //
-// GPU: the image is cut into 4 x 8 x 32 tiles (z contiguous); a block loads
-// a tile with a one-voxel halo into shared memory and relaxes it until it
-// stops changing, and a tile that changed wakes each neighbour across a
-// face where one of its voxels rose above the neighbour's value.  Two
-// schedules run the same relaxation:
-//  * rounds: woken tiles form the next round's work list; rounds end when
-//    a list is empty (or at the round cap).  One persistent cooperative
-//    grid with a grid-wide barrier between rounds for one large image; one
-//    ordinary launch per round in contexts that share the device with
-//    other streams, so that their kernels' blocks get in between rounds.
-//  * queue: one persistent ordinary launch over a work queue, no rounds and
-//    no barrier; the propagation ends when the queue is empty and no tile
-//    is being relaxed.  Used for batches and smaller images.
-// Everything other blocks write (the field, the lists, the queue, the
-// counters) is read with L2-coherent loads: the SM's L1 may hold a stale
-// line.
-#include <cooperative_groups.h>
-
-#include <cstring>
+// GPU: M follows from a maximum spanning forest, built by Boruvka rounds on
+// basins instead of voxels.
+//  * Order voxels by (value, index).  A voxel with a larger neighbour p (the
+//    largest one) has M[v] = min(val[v], M[p]): the edge to p is a largest
+//    one at v, so some best path starts with it.  Following p leads to a
+//    peak, along rising values, so M[v] = min(val[v], M[peak of v]): only
+//    the peaks' values are wanted.  Pointers are resolved inside a tile in
+//    shared memory first, then from tile to tile.
+//  * Basins (the voxels of one peak) are joined through their best edges: of
+//    all voxel pairs between a basin and others, and of its face voxels
+//    (edges to the outside, of the voxel's own value), the one of largest
+//    min(value).  With w its weight and D the basin beyond, M[C] = min(w,
+//    M[D]) by the same argument.  Every round hooks each root with an edge
+//    to the root beyond it (of two that choose each other the lower stays),
+//    and flattens the hooks with the running minimum, until no root has an
+//    edge; the outside is a root that never hooks, with M = infinity.
+// Ties between edges are broken by the edge's number, so hooks form no cycle.
+// After the first round the voxel pairs that still join different roots are
+// gathered into a list (or looked at again, if they outnumber it).
+//
+// The field was propagated before by relaxing 4 x 8 x 32 tiles until nothing
+// changed (about 20 activations a tile, 300 bytes a voxel, on a cooperative
+// grid or a work queue).  Here each voxel is read in a fixed number of passes
+// and everything is ordinary launches, so it runs beside other streams as it
+// is.
+#include <algorithm>
 #include <vector>
 
 #include "common.cuh"
 
-namespace cg = cooperative_groups;
-
 namespace {
 
-constexpr int TX = 4, TY = 8, TZ = 32;
-constexpr int kThreads = 256;
-constexpr int kPer = TX * TY * TZ / kThreads;   // voxels per thread
-constexpr int kInner = 96;                      // relaxation sweeps per activation
-// resident blocks per SM the register budget is sized for (measured on the
-// 512^3 blobs' trapping: 4 -> 36.7 ms, 5 -> 39.2 ms, 6 -> 43.8 ms)
-constexpr int kMinBlocks = 4;
-constexpr int kMaxRoundsDev = 1 << 16;
-// Single images of fewer tiles use the queue.  Measured with both schedules
-// (trapping of the 200^3 sphere pack, 8,750 tiles: rounds 3.50 ms, queue
-// 2.24 ms; of the 512^3 blobs, 131,072 tiles: 37.2 / 43.0 ms; the queue
-// then still stored whole tiles, before its atomic write-back of risen
-// voxels); the bound is the geometric midpoint of the two.
-constexpr int kQueueTiles = 32768;
-// a queue block that waits for work gives up, and stops the propagation
-// with an error status, once the grid has made no progress for this long
-constexpr unsigned long long kStallNs = 5000000000ull;
-// activation cap of the queue, in activations per tile (~20 in practice)
-constexpr int kQueueActsPerTile = 512;
+typedef unsigned long long u64;
 
-__device__ __forceinline__ unsigned long long mm_now_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
+constexpr int TX = 8, TY = 8, TZ = 32;          // tile of the pointer pass
+constexpr int kTileVox = TX * TY * TZ;
+constexpr int kThreads = 256;
+constexpr int kPer = kTileVox / kThreads;       // voxels per thread
+constexpr int kRoundsPerSync = 3;               // rounds launched between two looks at the flag
+constexpr int kMaxRoundsDev = 64;               // each round at least halves the roots with an edge
+constexpr uint32_t kBlocked = 0xffffffffu;
+constexpr uint32_t kPeak = 0x80000000u;         // label: kPeak | number of the peak
+
+// One image: its tiles and 32-voxel row segments are numbered globally.
+struct MMJob {
+    const int32_t *val;
+    uint32_t *M;            // pointer (linear index), then label, then the value
+    int nx, ny, nz, tx, ty, tz, face, segs;
+    int tile0, unit0;       // first tile / segment
+    int64_t vox0;           // voxels before this image
+};
+
+struct MMWork {
+    const MMJob *jobs;
+    int njobs, ntiles, nunits;
+    u64 *node;              // per basin: parent (low) and the smallest weight on the way there (high); [P] = outside
+    u64 *best;              // per root: weight << 33 | edge number of its best edge
+    int *ctr;               // [0] peaks, [1] listed edges, [2 + r] roots hooked in round r
+    int P;
+    int *ea, *eb, *ew;      // list of edges: two roots and the weight
+    int cap, listed;        // its length, and the entries in use (-1: not listed)
+};
 
 __device__ __forceinline__ int as_val(int v) { return v == -1 ? IBIP_INF32 : v; }
 
-// M = val on the unblocked voxels of the face, -1 elsewhere; a warp per
-// row (x, y), lanes along z, no per-voxel division
-__global__ void k_mm_init(const int32_t *__restrict__ val, int nx, int ny, int nz, int face, int32_t *M)
+template <class F>
+__device__ __forceinline__ int find_mm(int n, F first, int at)
 {
+    int lo = 0, hi = n;   // largest j with first(j) <= at
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (first(mid) <= at) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+__device__ __forceinline__ uint32_t parent_of(const MMWork &w, uint32_t c) { return (uint32_t)__ldcg(w.node + c); }
+
+// Pointers to the largest neighbour, resolved inside the tile: each voxel's
+// M gets the label of its peak or the index of the first voxel outside the
+// tile on the way there.
+__global__ void __launch_bounds__(kThreads) k_mm_tile(MMWork w)
+{
+    constexpr int HX = TX + 2, HY = TY + 2, HZ = TZ + 2, kHalo = HX * HY * HZ;
+    __shared__ int s_val[kHalo];
+    __shared__ unsigned short s_ptr[kTileVox];
+    __shared__ uint32_t s_tgt[kTileVox];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const MMJob J = w.jobs[find_mm(w.njobs, [&](int j) { return w.jobs[j].tile0; }, (int)blockIdx.x)];
+    const int t = (int)blockIdx.x - J.tile0;
+    const int bz = t % J.tz, by = (t / J.tz) % J.ty, bx = t / (J.tz * J.ty);
+    const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ;
+    for (int i = tid; i < kHalo; i += kThreads) {
+        const int hz = i % HZ, hy = (i / HZ) % HY, hx = i / (HZ * HY);
+        const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
+        int v = 0;
+        if (x >= 0 && y >= 0 && z >= 0 && x < J.nx && y < J.ny && z < J.nz)
+            v = as_val(__ldg(J.val + d_lin(x, y, z, J.ny, J.nz)));
+        s_val[i] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kPer; k++) {
+        const int i = tid + k * kThreads;
+        const int lz = i % TZ, ly = (i / TZ) % TY, lx = i / (TZ * TY);
+        const int h = ((lx + 1) * HY + ly + 1) * HZ + lz + 1;
+        const int v = s_val[h];
+        // the largest of the voxel and its neighbours by (value, index): the
+        // offsets in order of index are -x -y -z 0 +z +y +x
+        const int off[7] = {-HY * HZ, -HZ, -1, 0, 1, HZ, HY * HZ};
+        int b = -1, q = 3;
+#pragma unroll
+        for (int d = 0; d < 7; d++) {
+            const int u = s_val[h + off[d]];
+            if (u >= b) { b = u; q = d; }
+        }
+        int to = i;             // itself: a peak, blocked, or the way out of the tile
+        uint32_t tgt = kBlocked;
+        bool peak = false;
+        if (v != 0) {
+            if (q == 3) {
+                peak = true;
+            } else {
+                const int dx = q == 0 ? -1 : q == 6 ? 1 : 0, dy = q == 1 ? -1 : q == 5 ? 1 : 0;
+                const int dz = q == 2 ? -1 : q == 4 ? 1 : 0;
+                const int ux = lx + dx, uy = ly + dy, uz = lz + dz;
+                if (ux >= 0 && uy >= 0 && uz >= 0 && ux < TX && uy < TY && uz < TZ) to = (ux * TY + uy) * TZ + uz;
+                else tgt = (uint32_t)d_lin(x0 + ux, y0 + uy, z0 + uz, J.ny, J.nz);
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, peak);
+        if (m) {
+            int id = 0;
+            if (lane == 0) id = atomicAdd(w.ctr, __popc(m));
+            id = __shfl_sync(0xffffffffu, id, 0) + __popc(m & ((1u << lane) - 1));
+            if (peak) tgt = kPeak | (uint32_t)id;
+        }
+        s_ptr[i] = (unsigned short)to;
+        s_tgt[i] = tgt;
+    }
+    __syncthreads();
+    // follow the pointers to their ends inside the tile (they only rise, so
+    // there is no cycle); doubling, at most 11 passes for 2,048 voxels
+    for (int pass = 0; pass < 11; pass++) {
+        int ch = 0;
+#pragma unroll
+        for (int k = 0; k < kPer; k++) {
+            const int i = tid + k * kThreads;
+            const unsigned short p = s_ptr[i], q = s_ptr[p];
+            if (q != p) { s_ptr[i] = q; ch = 1; }
+        }
+        if (!__syncthreads_or(ch)) break;
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; k++) {
+        const int i = tid + k * kThreads;
+        const int lz = i % TZ, ly = (i / TZ) % TY, lx = i / (TZ * TY);
+        const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
+        if (x < J.nx && y < J.ny && z < J.nz) J.M[d_lin(x, y, z, J.ny, J.nz)] = s_tgt[s_ptr[i]];
+    }
+}
+
+// A warp's 32-voxel segment of a row: f(job, row, x, y, z, linear index, inside)
+template <class F>
+__device__ __forceinline__ void for_segments(const MMWork &w, F f)
+{
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    for (int u = blockIdx.x * wpb + (threadIdx.x >> 5); u < w.nunits; u += gridDim.x * wpb) {
+        const MMJob &J = w.jobs[find_mm(w.njobs, [&](int j) { return w.jobs[j].unit0; }, u)];
+        const int i = u - J.unit0, row = i / J.segs, z = (i - row * J.segs) * 32 + lane;
+        const int x = row / J.ny, y = row - x * J.ny;
+        f(J, x, y, z, (int64_t)row * J.nz + z, z < J.nz);
+    }
+}
+
+// the rest of the way to the peak, tile by tile
+__global__ void __launch_bounds__(kThreads) k_mm_label(MMWork w)
+{
+    for_segments(w, [&](const MMJob &J, int, int, int, int64_t v, bool in) {
+        if (!in) return;
+        uint32_t p = __ldcg(J.M + v);
+        if (p & kPeak) return;   // a label, or blocked
+        while (!(p & kPeak)) p = __ldcg(J.M + p);
+        __stcg(J.M + v, p);
+    });
+}
+
+__global__ void k_mm_nodes(MMWork w)
+{
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c <= w.P; c += gridDim.x * blockDim.x) {
+        w.node[c] = (u64)IBIP_INF32 << 32 | (uint32_t)c;
+        w.best[c] = 0ull;
+    }
+}
+
+__device__ __forceinline__ void offer(const MMWork &w, uint32_t c, u64 key)
+{
+    if (key > __ldcg(w.best + c)) atomicMax(w.best + c, key);
+}
+
+constexpr int kChunk = 64;   // list entries a warp takes at a time
+
+// Every voxel pair (the voxel and its +z, +y, +x neighbour) and every face
+// voxel as an edge.  LIST: those between different roots are appended to the
+// list, of each run of lanes with the same two roots only the largest; else
+// they are offered to the two roots (the outside, root P, takes none).
+template <bool LIST>
+__global__ void __launch_bounds__(kThreads) k_mm_pairs(MMWork w, int round)
+{
+    if (round > 0 && __ldcg(w.ctr + 2 + round - 1) == 0) return;
     const int lane = threadIdx.x & 31;
-    const int64_t nrows = (int64_t)nx * ny;
-    const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < nrows; row += wstride) {
-        const int x = (int)(row / ny), y = (int)(row - (int64_t)x * ny);
-        const bool row_on = (face == 0 && x == 0) || (face == 1 && x == nx - 1) || (face == 2 && y == 0) ||
-                            (face == 3 && y == ny - 1);
-        const int64_t b = row * nz;
-        for (int z = lane; z < nz; z += 32) {
-            const bool on = row_on || (face == 4 && z == 0) || (face == 5 && z == nz - 1);
-            int m = -1;
-            if (on) {
-                const int sv = val[b + z];
-                if (sv != 0) m = as_val(sv);
+    int lbase = 0, lleft = 0;   // list entries of the warp
+    for_segments(w, [&](const MMJob &J, int x, int y, int z, int64_t v, bool in) {
+        const uint32_t lb = in ? __ldcg(J.M + v) : kBlocked;
+        const int val = lb != kBlocked ? as_val(__ldg(J.val + v)) : 0;
+        uint32_t a = lb == kBlocked ? kBlocked : lb & ~kPeak;
+        const bool first = round == 0;
+        if (!first && a != kBlocked) a = parent_of(w, a);
+#pragma unroll
+        for (int d = 0; d < 4; d++) {
+            uint32_t b = kBlocked;
+            int wt = 0;
+            if (a != kBlocked) {
+                if (d < 3) {
+                    const bool ok = d == 0 ? z < J.nz - 1 : d == 1 ? y < J.ny - 1 : x < J.nx - 1;
+                    const int64_t u = v + (d == 0 ? 1 : d == 1 ? (int64_t)J.nz : (int64_t)J.ny * J.nz);
+                    if (ok) {
+                        const uint32_t lu = __ldcg(J.M + u);
+                        if (lu != kBlocked && lu != lb) {
+                            b = lu & ~kPeak;
+                            if (!first) b = parent_of(w, b);
+                            wt = min(val, as_val(__ldg(J.val + u)));
+                        }
+                    }
+                } else if (d_on_face(x, y, z, J.nx, J.ny, J.nz, J.face)) {
+                    b = (uint32_t)w.P;
+                    wt = val;
+                }
             }
-            M[b + z] = m;
+            bool edge = b != kBlocked && a != b;
+            if (LIST) {
+                if (!__any_sync(0xffffffffu, edge)) continue;
+                // runs of the same two roots: the largest weight, kept by the
+                // last lane of the run
+                const uint32_t pa = __shfl_up_sync(0xffffffffu, a, 1), pb = __shfl_up_sync(0xffffffffu, b, 1);
+                const bool cont = __shfl_up_sync(0xffffffffu, (int)edge, 1) && lane > 0 && edge && pa == a && pb == b;
+                const unsigned heads = __ballot_sync(0xffffffffu, !cont);
+                const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, wt, o);
+                    if (lane - o >= start) wt = max(wt, t);
+                }
+                edge = edge && (lane == 31 || ((heads >> (lane + 1)) & 1u));
+                const unsigned m = __ballot_sync(0xffffffffu, edge);
+                const int need = __popc(m), k = __popc(m & ((1u << lane) - 1));
+                int pos = lbase + k;
+                if (lleft < need) {
+                    int nb = 0;
+                    if (lane == 0) nb = atomicAdd(w.ctr + 1, kChunk);
+                    nb = __shfl_sync(0xffffffffu, nb, 0) - lleft;
+                    if (k >= lleft) pos = nb + k;
+                    lbase = nb;
+                    lleft += kChunk;
+                }
+                if (edge && pos < w.cap) {
+                    w.ea[pos] = (int)a;
+                    w.eb[pos] = (int)b;
+                    w.ew[pos] = wt;
+                }
+                lbase += need;
+                lleft -= need;
+            } else if (edge) {
+                const u64 key = (u64)(uint32_t)wt << 33 | (u64)(4 * (J.vox0 + v) + d);
+                if (a != (uint32_t)w.P) offer(w, a, key);
+                if (b != (uint32_t)w.P) offer(w, b, key);
+            }
         }
+    });
+    if (LIST)   // the entries left over are no edges
+        for (int i = lane; i < lleft; i += 32)
+            if (lbase + i < w.cap) w.ea[lbase + i] = w.eb[lbase + i] = 0;
+}
+
+// the listed edges: ends moved to their roots, then offered
+__global__ void __launch_bounds__(kThreads) k_mm_edges(MMWork w, int round)
+{
+    if (__ldcg(w.ctr + 2 + round - 1) == 0) return;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < w.listed; e += gridDim.x * blockDim.x) {
+        int a = w.ea[e], b = w.eb[e];
+        if (a == b) continue;
+        a = (int)parent_of(w, (uint32_t)a);
+        b = (int)parent_of(w, (uint32_t)b);
+        w.ea[e] = a;
+        w.eb[e] = b;
+        if (a == b) continue;
+        const u64 key = (u64)(uint32_t)w.ew[e] << 33 | (u64)e;
+        if (a != w.P) offer(w, (uint32_t)a, key);
+        if (b != w.P) offer(w, (uint32_t)b, key);
     }
 }
 
-// One image of a (possibly batched) propagation; its tiles are numbered
-// tile0 .. tile0 + tx*ty*tz - 1 in the global tile space.
-struct MMJob {
-    const int32_t *val;
-    int32_t *M;
-    int nx, ny, nz, tx, ty, tz, face, tile0;
-};
-
-// tiles touching each image's face start the first round's list
-__global__ void k_mm_seed(const MMJob *__restrict__ jobs, int njobs, int ntot, int *list, int *count, int *mark)
+// each root hooks to the root beyond its best edge
+__global__ void __launch_bounds__(kThreads) k_mm_hook(MMWork w, int round)
 {
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ntot; g += gridDim.x * blockDim.x) {
-        int lo = 0, hi = njobs;   // job: largest j with tile0 <= g
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (jobs[mid].tile0 <= g) lo = mid; else hi = mid;
+    if (round > 0 && __ldcg(w.ctr + 2 + round - 1) == 0) return;
+    const int lane = threadIdx.x & 31;
+    for (int c0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; c0 < w.P; c0 += gridDim.x * blockDim.x) {
+        const int c = c0 + lane;
+        bool hook = false;
+        if (c < w.P && (uint32_t)w.node[c] == (uint32_t)c) {
+            const u64 key = __ldcg(w.best + c);
+            if (key) {
+                const u64 id = key & ((1ull << 33) - 1);
+                uint32_t a, b;
+                if (w.listed >= 0) {
+                    a = (uint32_t)w.ea[id];
+                    b = (uint32_t)w.eb[id];
+                } else {
+                    const int64_t gv = (int64_t)(id >> 2);
+                    const int d = (int)(id & 3);
+                    int lo = 0, hi = w.njobs;
+                    while (hi - lo > 1) {
+                        const int mid = (lo + hi) >> 1;
+                        if (w.jobs[mid].vox0 <= gv) lo = mid; else hi = mid;
+                    }
+                    const MMJob &J = w.jobs[lo];
+                    const int64_t v = gv - J.vox0;
+                    a = __ldcg(J.M + v) & ~kPeak;
+                    b = d == 3 ? (uint32_t)w.P
+                               : __ldcg(J.M + v + (d == 0 ? 1 : d == 1 ? (int64_t)J.nz : (int64_t)J.ny * J.nz)) & ~kPeak;
+                    if (round > 0) {   // c is one of the two roots: the labels' parents before this round's hooks
+                        const uint32_t pa = parent_of(w, a), pb = d == 3 ? b : parent_of(w, b);
+                        a = a == (uint32_t)c || pa == (uint32_t)c ? (uint32_t)c : pa;
+                        b = b == (uint32_t)c || pb == (uint32_t)c ? (uint32_t)c : pb;
+                    }
+                }
+                const uint32_t o = a == (uint32_t)c ? b : a;
+                // (o == c: the other end has hooked to c just now)
+                hook = o != (uint32_t)c && !(o != (uint32_t)w.P && __ldcg(w.best + o) == key && (uint32_t)c < o);
+                if (hook) __stcg(w.node + c, (key >> 33) << 32 | o);
+            }
         }
-        const MMJob &J = jobs[lo];
-        const int t = g - J.tile0;
-        const int bz = t % J.tz, by = (t / J.tz) % J.ty, bx = t / (J.tz * J.ty);
-        bool on = false;
-        switch (J.face) {
-        case 0: on = bx == 0; break;
-        case 1: on = bx == J.tx - 1; break;
-        case 2: on = by == 0; break;
-        case 3: on = by == J.ty - 1; break;
-        case 4: on = bz == 0; break;
-        default: on = bz == J.tz - 1; break;
-        }
-        if (on) {
-            mark[g] = 0;
-            list[atomicAdd(count, 1)] = g;
-        }
+        const unsigned m = __ballot_sync(0xffffffffu, hook);
+        if (m && lane == 0) atomicAdd(w.ctr + 2 + round, __popc(m));
     }
 }
 
-struct MMArgs {
-    const MMJob *jobs;
-    int njobs;
-    int *list0, *list1;   // work lists of global tile ids, alternating by round
-    int *count, *head;    // per-round list sizes and take counters [max_rounds + 2]
-    int *mark;            // per tile: last round it was queued for
-    int *status;          // [0] rounds run, [1] 1 if the round cap was hit, [2] relaxation sweeps
-    int max_rounds;
-};
-
-// Claims and relaxes the tiles of round r's list until the list is drained.
-// A tile queues a neighbour for round r + 1 only where one of its face
-// voxels rose in this activation above the neighbour's value across that
-// face (as loaded): M only grows, so no other neighbour can improve.  In
-// round 0 the seeded values count as risen.
-__device__ void mm_round(const MMArgs &a, int r, int32_t (*sM)[TY + 2][TZ + 2], int *s_tile, int *s_wake)
+// hooks flattened: every basin points at its root, with the smallest weight
+// on the way (the pair is one 64-bit word, so a half-done neighbour reads
+// consistently)
+__global__ void __launch_bounds__(kThreads) k_mm_flatten(MMWork w, int round)
 {
-    const int cnt = __ldcg(a.count + r);
-    const int *list = (r & 1) ? a.list1 : a.list0;
-    int *next = (r & 1) ? a.list0 : a.list1;
-    // thread 0 claims one tile ahead: the claim is issued when the current
-    // tile starts and its list entry read after the relaxation, so neither
-    // round trip lies on the path between two tiles
-    int next_g = -1;
-    if (threadIdx.x == 0) {
-        const int q = atomicAdd(&a.head[r], 1);
-        next_g = q < cnt ? __ldcg(list + q) : -1;
-    }
-    for (;;) {
-        if (threadIdx.x == 0) *s_tile = next_g;
-        __syncthreads();
-        const int g = *s_tile;
-        if (g < 0) break;
-        int q_next = 0;
-        if (threadIdx.x == 0) q_next = atomicAdd(&a.head[r], 1);
-        int lo = 0, hi = a.njobs;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(&a.jobs[mid].tile0) <= g) lo = mid; else hi = mid;
+    if (__ldcg(w.ctr + 2 + round) == 0) return;
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < w.P; c += gridDim.x * blockDim.x) {
+        const u64 x = __ldcg(w.node + c);
+        uint32_t p = (uint32_t)x, m = (uint32_t)(x >> 32);
+        w.best[c] = 0ull;
+        if (p == (uint32_t)c) continue;
+        for (;;) {
+            const u64 y = __ldcg(w.node + p);
+            if ((uint32_t)y == p) break;
+            m = min(m, (uint32_t)(y >> 32));
+            p = (uint32_t)y;
         }
-        const MMJob J = a.jobs[lo];
-        const int t = g - J.tile0;
-        const int bz = t % J.tz, by = (t / J.tz) % J.ty, bx = t / (J.tz * J.ty);
-        const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ;
-        // the tile's values and the field on the tile plus a one-voxel halo:
-        // every load is issued before the first store to shared memory
-        int sval[kPer], lx[kPer], ly[kPer], lz[kPer];
-#pragma unroll
-        for (int k = 0; k < kPer; k++) {
-            const int i = threadIdx.x + k * kThreads;
-            lz[k] = i % TZ; ly[k] = (i / TZ) % TY; lx[k] = i / (TZ * TY);
-            const int x = x0 + lx[k], y = y0 + ly[k], z = z0 + lz[k];
-            sval[k] = (x < J.nx && y < J.ny && z < J.nz) ? J.val[d_lin(x, y, z, J.ny, J.nz)] : 0;
-        }
-        constexpr int kHalo = (TX + 2) * (TY + 2) * (TZ + 2);
-        constexpr int kHaloPer = (kHalo + kThreads - 1) / kThreads;
-        int hv[kHaloPer];
-#pragma unroll
-        for (int u = 0; u < kHaloPer; u++) {
-            const int i = threadIdx.x + u * kThreads;
-            const int hz = i % (TZ + 2), hy = (i / (TZ + 2)) % (TY + 2), hx = i / ((TZ + 2) * (TY + 2));
-            const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
-            hv[u] = -1;
-            if (i < kHalo && x >= 0 && y >= 0 && z >= 0 && x < J.nx && y < J.ny && z < J.nz)
-                hv[u] = __ldcg(J.M + d_lin(x, y, z, J.ny, J.nz));
-        }
-        int32_t *sflat = &sM[0][0][0];
-#pragma unroll
-        for (int u = 0; u < kHaloPer; u++) {
-            const int i = threadIdx.x + u * kThreads;
-            if (i < kHalo) sflat[i] = hv[u];
-        }
-#pragma unroll
-        for (int k = 0; k < kPer; k++) sval[k] = as_val(sval[k]);
-        if (threadIdx.x < 6) s_wake[threadIdx.x] = 0;
-        __syncthreads();
-        int mold[kPer];
-#pragma unroll
-        for (int k = 0; k < kPer; k++) mold[k] = r == 0 ? -1 : sM[lx[k] + 1][ly[k] + 1][lz[k] + 1];
-        bool any = false, conv = false;
-        int sweeps = 0;
-        for (int it = 0; it < kInner; it++) {
-            sweeps++;
-            int ch = 0;
-#pragma unroll
-            for (int k = 0; k < kPer; k++) {
-                if (sval[k] == 0) continue;
-                const int hx = lx[k] + 1, hy = ly[k] + 1, hz = lz[k] + 1;
-                const int b = max(max(max(sM[hx - 1][hy][hz], sM[hx + 1][hy][hz]), max(sM[hx][hy - 1][hz], sM[hx][hy + 1][hz])),
-                                  max(sM[hx][hy][hz - 1], sM[hx][hy][hz + 1]));
-                const int nv = min(b, sval[k]);
-                if (nv > sM[hx][hy][hz]) { sM[hx][hy][hz] = nv; ch = 1; }
-            }
-            if (!__syncthreads_or(ch)) { conv = true; break; }
-            any = true;
-        }
-        if (threadIdx.x == 0) {
-            atomicAdd(a.status + 2, sweeps);
-            next_g = q_next < cnt ? __ldcg(list + q_next) : -1;
-        }
-#pragma unroll
-        for (int k = 0; k < kPer; k++) {
-            if (sval[k] == 0) continue;
-            const int hx = lx[k] + 1, hy = ly[k] + 1, hz = lz[k] + 1;
-            const int mv = sM[hx][hy][hz];
-            if (mv <= mold[k]) continue;   // not risen here
-            if (lx[k] == 0 && mv > sM[0][hy][hz]) s_wake[0] = 1;
-            if (lx[k] == TX - 1 && mv > sM[TX + 1][hy][hz]) s_wake[1] = 1;
-            if (ly[k] == 0 && mv > sM[hx][0][hz]) s_wake[2] = 1;
-            if (ly[k] == TY - 1 && mv > sM[hx][TY + 1][hz]) s_wake[3] = 1;
-            if (lz[k] == 0 && mv > sM[hx][hy][0]) s_wake[4] = 1;
-            if (lz[k] == TZ - 1 && mv > sM[hx][hy][TZ + 1]) s_wake[5] = 1;
-        }
-        __syncthreads();
-        if (any) {
-#pragma unroll
-            for (int k = 0; k < kPer; k++) {
-                const int x = x0 + lx[k], y = y0 + ly[k], z = z0 + lz[k];
-                if (x < J.nx && y < J.ny && z < J.nz && sval[k] != 0)
-                    J.M[d_lin(x, y, z, J.ny, J.nz)] = sM[lx[k] + 1][ly[k] + 1][lz[k] + 1];
-            }
-        }
-        if (threadIdx.x < 7) {   // one lane per neighbour (6) and the tile itself: the atomics overlap
-            const int q = threadIdx.x, nr = r + 1;
-            int nb = -1;
-            switch (q) {
-            case 0: if (bx > 0 && s_wake[0]) nb = g - J.tz * J.ty; break;
-            case 1: if (bx < J.tx - 1 && s_wake[1]) nb = g + J.tz * J.ty; break;
-            case 2: if (by > 0 && s_wake[2]) nb = g - J.tz; break;
-            case 3: if (by < J.ty - 1 && s_wake[3]) nb = g + J.tz; break;
-            case 4: if (bz > 0 && s_wake[4]) nb = g - 1; break;
-            case 5: if (bz < J.tz - 1 && s_wake[5]) nb = g + 1; break;
-            default: if (!conv) nb = g; break;
-            }
-            if (nb >= 0 && atomicMax(&a.mark[nb], nr) < nr) next[atomicAdd(&a.count[nr], 1)] = nb;
-        }
-        __syncthreads();
+        __stcg(w.node + c, (u64)m << 32 | p);
     }
 }
 
-// All rounds in one cooperative launch, a grid barrier between rounds.
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_mm_persistent(MMArgs a)
+// M = min(value, the smallest weight to the outside), -1 where it is not reached
+__global__ void __launch_bounds__(kThreads) k_mm_value(MMWork w)
 {
-    cg::grid_group grid = cg::this_grid();
-    __shared__ int32_t sM[TX + 2][TY + 2][TZ + 2];
-    __shared__ int s_tile, s_wake[6];
-    int r = 0;
-    for (;; r++) {
-        if (__ldcg(a.count + r) == 0 || r >= a.max_rounds) break;
-        mm_round(a, r, sM, &s_tile, s_wake);
-        __threadfence();
-        grid.sync();
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        a.status[0] = r;
-        a.status[1] = (r >= a.max_rounds && __ldcg(a.count + r) != 0) ? 1 : 0;
-    }
-}
-
-// One round per launch: for contexts whose kernels share the device with
-// other streams (a cooperative grid could not be made resident beside them).
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_mm_round(MMArgs a, int r)
-{
-    __shared__ int32_t sM[TX + 2][TY + 2][TZ + 2];
-    __shared__ int s_tile, s_wake[6];
-    if (r >= a.max_rounds || __ldcg(a.count + r) == 0) return;
-    mm_round(a, r, sM, &s_tile, s_wake);
-}
-
-// The work queue: a ring of entries (tile id, bit 30 = queued as a seed; -1 =
-// empty slot) with monotone head and tail counters.  A block takes a
-// ticket (head) before it needs the tile and waits, when it does, for the
-// push that fills its slot.  A tile is pushed only when its flag goes from
-// 0 to 1 and the flag is cleared when it is taken, so the ring never holds
-// more than ntiles entries; its capacity adds a slot per block for the
-// tickets not yet filled.
-struct MMQ {
-    const MMJob *jobs;
-    int njobs;
-    int *ring;                    // [cap]
-    int *queued;                  // per tile: 1 while in the ring
-    unsigned long long *head, *tail;
-    int *pending;                 // tiles in the ring or being relaxed
-    unsigned long long *acts;     // tile activations so far (progress)
-    int *sweeps;                  // relaxation sweeps (diagnostics)
-    int *stop;                    // 1: activation cap reached, 2: no progress
-    long long max_acts;
-    int cap;
-};
-
-constexpr int kSeedBit = 1 << 30;
-
-// Queue tile g unless it is waiting already; a seed tile's first relaxation
-// counts every voxel as risen (its face values were set before it ran).
-// pending counts the tile before it can be taken, so the count never
-// reaches 0 while work remains.
-__device__ __forceinline__ void mmq_push(const MMQ &Q, int g, bool seed)
-{
-    if (atomicCAS(Q.queued + g, 0, 1) != 0) return;
-    atomicAdd(Q.pending, 1);
-    __threadfence();
-    const unsigned long long t = atomicAdd(Q.tail, 1ull);
-    *(volatile int *)(Q.ring + (int)(t % (unsigned long long)Q.cap)) = g | (seed ? kSeedBit : 0);
-}
-
-// The tile of ticket h (*seed: queued as a seed), or -1 once the
-// propagation is over (nothing queued or being relaxed, so no push will
-// come) or stopped.  Only the ticket's holder reads its slot.
-__device__ int mmq_take(const MMQ &Q, unsigned long long h, bool *seed)
-{
-    volatile int *slot = Q.ring + (int)(h % (unsigned long long)Q.cap);
-    unsigned long long seen = ~0ull, since = 0;
-    for (;;) {
-        if (*(volatile int *)Q.stop) return -1;
-        const int raw = *slot;
-        if (raw >= 0) {
-            *slot = -1;
-            const int g = raw & (kSeedBit - 1);
-            *seed = (raw & kSeedBit) != 0;
-            atomicAnd(Q.queued + g, 0);
-            __threadfence();
-            return g;
+    for_segments(w, [&](const MMJob &J, int, int, int, int64_t v, bool in) {
+        if (!in) return;
+        const uint32_t lb = __ldcg(J.M + v);
+        int m = -1;
+        if (lb != kBlocked) {
+            const u64 x = __ldcg(w.node + (lb & ~kPeak));
+            if ((uint32_t)x == (uint32_t)w.P) m = min(as_val(__ldg(J.val + v)), (int)(x >> 32));
         }
-        if (*(volatile int *)Q.pending == 0) return -1;
-        // blocks still relaxing may queue more; give up only when the
-        // whole grid has made no progress for kStallNs
-        const unsigned long long a = *(volatile unsigned long long *)Q.acts;
-        const unsigned long long now = mm_now_ns();
-        if (a != seen) { seen = a; since = now; }
-        else if (now - since > kStallNs) { atomicExch(Q.stop, 2); return -1; }
-        __nanosleep(64);
-    }
-}
-
-// The tile of ticket h if its slot is filled already (returns false, and
-// takes nothing, otherwise).
-__device__ __forceinline__ bool mmq_try_take(const MMQ &Q, unsigned long long h, int *g, bool *seed)
-{
-    volatile int *slot = Q.ring + (int)(h % (unsigned long long)Q.cap);
-    const int raw = *slot;
-    if (raw < 0) return false;
-    *slot = -1;
-    *g = raw & (kSeedBit - 1);
-    *seed = (raw & kSeedBit) != 0;
-    atomicAnd(Q.queued + *g, 0);
-    __threadfence();
-    return true;
-}
-
-// tiles touching each image's face are queued first (queue schedule)
-__global__ void k_mm_qseed(MMQ Q, int ntot)
-{
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ntot; g += gridDim.x * blockDim.x) {
-        int lo = 0, hi = Q.njobs;   // job: largest j with tile0 <= g
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (Q.jobs[mid].tile0 <= g) lo = mid; else hi = mid;
-        }
-        const MMJob &J = Q.jobs[lo];
-        const int t = g - J.tile0;
-        const int bz = t % J.tz, by = (t / J.tz) % J.ty, bx = t / (J.tz * J.ty);
-        bool on = false;
-        switch (J.face) {
-        case 0: on = bx == 0; break;
-        case 1: on = bx == J.tx - 1; break;
-        case 2: on = by == 0; break;
-        case 3: on = by == J.ty - 1; break;
-        case 4: on = bz == 0; break;
-        default: on = bz == J.tz - 1; break;
-        }
-        if (on) mmq_push(Q, g, true);
-    }
-}
-
-// One persistent launch: each block relaxes tiles from the queue until the
-// propagation is over.  Thread 0 takes the ticket of the block's next tile
-// when the current one starts, so that atomic is off the path between tiles.
-// A tile queues a neighbour only where one of its face voxels rose in this
-// relaxation above the neighbour's value across that face (as loaded): M
-// only grows, so no other neighbour can improve.  A seed tile's first
-// relaxation counts its face values as risen.
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_mm_queue(MMQ Q)
-{
-    __shared__ int32_t sM[TX + 2][TY + 2][TZ + 2];
-    __shared__ int s_tile, s_seed, s_wake[6];
-    int next_g = -1, my_acts = 0, my_sweeps = 0;
-    bool next_seed = false;
-    if (threadIdx.x == 0) next_g = mmq_take(Q, atomicAdd(Q.head, 1ull), &next_seed);
-    for (;;) {
-        if (threadIdx.x == 0) { s_tile = next_g; s_seed = next_seed ? 1 : 0; }
-        __syncthreads();
-        const int g = s_tile;
-        const bool seed = s_seed != 0;
-        if (g < 0) {
-            if (threadIdx.x == 0 && my_acts) {
-                atomicAdd(Q.sweeps, my_sweeps);
-                atomicAdd(Q.acts, (unsigned long long)my_acts);
-            }
-            break;
-        }
-        unsigned long long ticket = 0;
-        if (threadIdx.x == 0) ticket = atomicAdd(Q.head, 1ull);
-        int lo = 0, hi = Q.njobs;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (__ldg(&Q.jobs[mid].tile0) <= g) lo = mid; else hi = mid;
-        }
-        const MMJob J = Q.jobs[lo];
-        const int t = g - J.tile0;
-        const int bz = t % J.tz, by = (t / J.tz) % J.ty, bx = t / (J.tz * J.ty);
-        const int x0 = bx * TX, y0 = by * TY, z0 = bz * TZ;
-        // the tile's values and the field on the tile plus a one-voxel halo:
-        // every load is issued before the first store to shared memory
-        int sval[kPer], lx[kPer], ly[kPer], lz[kPer];
-#pragma unroll
-        for (int k = 0; k < kPer; k++) {
-            const int i = threadIdx.x + k * kThreads;
-            lz[k] = i % TZ; ly[k] = (i / TZ) % TY; lx[k] = i / (TZ * TY);
-            const int x = x0 + lx[k], y = y0 + ly[k], z = z0 + lz[k];
-            sval[k] = (x < J.nx && y < J.ny && z < J.nz) ? J.val[d_lin(x, y, z, J.ny, J.nz)] : 0;
-        }
-        constexpr int kHalo = (TX + 2) * (TY + 2) * (TZ + 2);
-        constexpr int kHaloPer = (kHalo + kThreads - 1) / kThreads;
-        int hv[kHaloPer];
-#pragma unroll
-        for (int u = 0; u < kHaloPer; u++) {
-            const int i = threadIdx.x + u * kThreads;
-            const int hz = i % (TZ + 2), hy = (i / (TZ + 2)) % (TY + 2), hx = i / ((TZ + 2) * (TY + 2));
-            const int x = x0 + hx - 1, y = y0 + hy - 1, z = z0 + hz - 1;
-            hv[u] = -1;
-            if (i < kHalo && x >= 0 && y >= 0 && z >= 0 && x < J.nx && y < J.ny && z < J.nz)
-                hv[u] = __ldcg(J.M + d_lin(x, y, z, J.ny, J.nz));
-        }
-        int32_t *sflat = &sM[0][0][0];
-#pragma unroll
-        for (int u = 0; u < kHaloPer; u++) {
-            const int i = threadIdx.x + u * kThreads;
-            if (i < kHalo) sflat[i] = hv[u];
-        }
-#pragma unroll
-        for (int k = 0; k < kPer; k++) sval[k] = as_val(sval[k]);
-        if (threadIdx.x < 6) s_wake[threadIdx.x] = 0;
-        __syncthreads();
-        int mold[kPer];
-#pragma unroll
-        for (int k = 0; k < kPer; k++) mold[k] = seed ? -1 : sM[lx[k] + 1][ly[k] + 1][lz[k] + 1];
-        bool any = false, conv = false;
-        int sweeps = 0;
-        for (int it = 0; it < kInner; it++) {
-            sweeps++;
-            int ch = 0;
-#pragma unroll
-            for (int k = 0; k < kPer; k++) {
-                if (sval[k] == 0) continue;
-                const int hx = lx[k] + 1, hy = ly[k] + 1, hz = lz[k] + 1;
-                const int b = max(max(max(sM[hx - 1][hy][hz], sM[hx + 1][hy][hz]), max(sM[hx][hy - 1][hz], sM[hx][hy + 1][hz])),
-                                  max(sM[hx][hy][hz - 1], sM[hx][hy][hz + 1]));
-                const int nv = min(b, sval[k]);
-                if (nv > sM[hx][hy][hz]) { sM[hx][hy][hz] = nv; ch = 1; }
-            }
-            if (!__syncthreads_or(ch)) { conv = true; break; }
-            any = true;
-        }
-        // the next tile, if its push has come already: taken while this
-        // one's results are written
-        bool got = false;
-        if (threadIdx.x == 0) got = mmq_try_take(Q, ticket, &next_g, &next_seed);
-#pragma unroll
-        for (int k = 0; k < kPer; k++) {
-            if (sval[k] == 0) continue;
-            const int hx = lx[k] + 1, hy = ly[k] + 1, hz = lz[k] + 1;
-            const int mv = sM[hx][hy][hz];
-            if (mv <= mold[k]) continue;   // not risen here
-            if (lx[k] == 0 && mv > sM[0][hy][hz]) s_wake[0] = 1;
-            if (lx[k] == TX - 1 && mv > sM[TX + 1][hy][hz]) s_wake[1] = 1;
-            if (ly[k] == 0 && mv > sM[hx][0][hz]) s_wake[2] = 1;
-            if (ly[k] == TY - 1 && mv > sM[hx][TY + 1][hz]) s_wake[3] = 1;
-            if (lz[k] == 0 && mv > sM[hx][hy][0]) s_wake[4] = 1;
-            if (lz[k] == TZ - 1 && mv > sM[hx][hy][TZ + 1]) s_wake[5] = 1;
-        }
-        // A tile woken again while it is being relaxed can be taken by
-        // another block before this one finishes, so two blocks may relax
-        // it at once; the one that loaded older values must not overwrite
-        // the other's.  Only risen voxels are written, by atomic maximum:
-        // the field never falls.
-        if (any) {
-#pragma unroll
-            for (int k = 0; k < kPer; k++) {
-                const int x = x0 + lx[k], y = y0 + ly[k], z = z0 + lz[k];
-                const int mv = sM[lx[k] + 1][ly[k] + 1][lz[k] + 1];
-                if (x < J.nx && y < J.ny && z < J.nz && sval[k] != 0 && mv > mold[k])
-                    atomicMax(J.M + d_lin(x, y, z, J.ny, J.nz), mv);
-            }
-        }
-        // the field's stores are visible before any neighbour is queued
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x < 7) {   // one lane per neighbour (6) and the tile itself: the pushes overlap
-            const int q = threadIdx.x;
-            int nb = -1;
-            switch (q) {
-            case 0: if (bx > 0 && s_wake[0]) nb = g - J.tz * J.ty; break;
-            case 1: if (bx < J.tx - 1 && s_wake[1]) nb = g + J.tz * J.ty; break;
-            case 2: if (by > 0 && s_wake[2]) nb = g - J.tz; break;
-            case 3: if (by < J.ty - 1 && s_wake[3]) nb = g + J.tz; break;
-            case 4: if (bz > 0 && s_wake[4]) nb = g - 1; break;
-            case 5: if (bz < J.tz - 1 && s_wake[5]) nb = g + 1; break;
-            default: if (!conv) nb = g; break;
-            }
-            if (nb >= 0) mmq_push(Q, nb, false);
-            __threadfence();
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            // counters in batches of 16 tiles (the activation cap and the
-            // stall watch need no finer grain)
-            my_sweeps += sweeps;
-            if (++my_acts == 16) {
-                atomicAdd(Q.sweeps, my_sweeps);
-                if ((long long)atomicAdd(Q.acts, 16ull) + 16 >= Q.max_acts) atomicExch(Q.stop, 1);
-                my_acts = my_sweeps = 0;
-            }
-            atomicSub(Q.pending, 1);   // this tile is done; its pushes were counted first
-            if (!got) next_g = mmq_take(Q, ticket, &next_seed);
-        }
-    }
+        J.M[v] = (uint32_t)m;
+    });
 }
 
 }  // namespace
 
-namespace {
-
-// The queue schedule over the jobs' tiles (0 .. nt-1).
-int mm_run_queue(ibip_ctx *ctx, int n, const std::vector<MMJob> &J, int nt, int rounds)
+// The jobs' voxels together stay below 2^31.
+static int mm_group(ibip_ctx *ctx, int n, const IbipMaximinJob *jobs)
 {
-    cudaStream_t s = ctx->stream;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mm_queue, kThreads, 0) != cudaSuccess ||
-        per_sm < 1) {
-        cudaGetLastError();
-        return IBIP_ERR_CUDA;
-    }
-    int grid = ctx->sm_count * per_sm;
-    if (grid > nt) grid = nt;
-    const int cap = nt + grid + 64;
-    // layout: jobs | head tail acts (u64) pending sweeps stop (int) | ring[cap] queued[nt]
-    const size_t jb = ((size_t)n * sizeof(MMJob) + 255) & ~(size_t)255;
-    const size_t cb = 64;
-    char *w0 = (char *)ibip_scratch(ctx, SC_TILE, jb + cb + ((size_t)cap + nt) * sizeof(int));
-    if (!w0) return IBIP_ERR_OOM;
-    MMQ Q;
-    Q.jobs = (MMJob *)w0; Q.njobs = n;
-    unsigned long long *c64 = (unsigned long long *)(w0 + jb);
-    Q.head = c64; Q.tail = c64 + 1; Q.acts = c64 + 2;
-    int *c32 = (int *)(c64 + 3);
-    Q.pending = c32; Q.sweeps = c32 + 1; Q.stop = c32 + 2;
-    Q.ring = (int *)(w0 + jb + cb); Q.queued = Q.ring + cap;
-    Q.cap = cap;
-    Q.max_acts = (long long)(rounds < kQueueActsPerTile ? rounds : kQueueActsPerTile) * nt;
-    ibip_prof_begin(ctx, IBIP_K_MAXIMIN);
-    cudaMemcpyAsync((void *)Q.jobs, J.data(), (size_t)n * sizeof(MMJob), cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(w0 + jb, 0, cb, s);                              // counters
-    cudaMemsetAsync(Q.ring, 0xff, (size_t)cap * sizeof(int), s);     // -1: empty slots
-    cudaMemsetAsync(Q.queued, 0, (size_t)nt * sizeof(int), s);
+    std::vector<MMJob> J(n);
+    int64_t vox = 0, tiles = 0, units = 0;
     for (int j = 0; j < n; j++) {
-        k_mm_init<<<ctx->sm_count * 4, 256, 0, s>>>(J[j].val, J[j].nx, J[j].ny, J[j].nz, J[j].face, J[j].M);
-        IBIP_LAUNCH(ctx);
+        const ibip_dims d = jobs[j].d;
+        MMJob &q = J[j];
+        q.val = jobs[j].val;
+        q.M = (uint32_t *)jobs[j].M;
+        q.nx = d.nx; q.ny = d.ny; q.nz = d.nz; q.face = jobs[j].face;
+        q.tx = (d.nx + TX - 1) / TX; q.ty = (d.ny + TY - 1) / TY; q.tz = (d.nz + TZ - 1) / TZ;
+        q.segs = (d.nz + 31) / 32;
+        q.tile0 = (int)tiles; q.unit0 = (int)units; q.vox0 = vox;
+        tiles += (int64_t)q.tx * q.ty * q.tz;
+        units += (int64_t)d.nx * d.ny * q.segs;
+        vox += nvox(d);
     }
-    k_mm_qseed<<<(nt + 255) / 256, 256, 0, s>>>(Q, nt);
-    IBIP_LAUNCH(ctx);
-    // a server slot issues it on its high-priority stream, beside the wide
-    // kernels of the other jobs
+    if (tiles >= (1ll << 31) || units >= (1ll << 31)) return IBIP_ERR_ARG;
+    cudaStream_t s = ctx->stream;
+    const size_t jb = ((size_t)n * sizeof(MMJob) + 255) & ~(size_t)255;
+    const size_t cb = (2 + kMaxRoundsDev) * sizeof(int);
+    char *t = (char *)ibip_scratch(ctx, SC_TILE, jb + cb);
+    if (!t) return IBIP_ERR_OOM;
+    MMWork w = {};
+    w.jobs = (const MMJob *)t;
+    w.njobs = n;
+    w.ntiles = (int)tiles;
+    w.nunits = (int)units;
+    w.ctr = (int *)(t + jb);
+    w.listed = -1;
+    ibip_prof_begin(ctx, IBIP_K_MAXIMIN);
+    cudaMemcpyAsync(t, J.data(), (size_t)n * sizeof(MMJob), cudaMemcpyHostToDevice, s);
+    cudaMemsetAsync(w.ctr, 0, cb, s);
     if (ctx->stream_inv) {
+        // server slot: on the high-priority stream, ahead of the wide kernels
+        // of the other jobs
         if (cudaEventRecord(ctx->ev_inv, s) != cudaSuccess ||
             cudaStreamWaitEvent(ctx->stream_inv, ctx->ev_inv, 0) != cudaSuccess)
             return ibip_cuda_status(cudaGetLastError());
         s = ctx->stream_inv;
     }
-    k_mm_queue<<<grid, kThreads, 0, s>>>(Q);
-    IBIP_LAUNCH(ctx);
+    const int wide = (int)std::min<int64_t>((units + kThreads / 32 - 1) / (kThreads / 32), (int64_t)ctx->sm_count * 32);
+    k_mm_tile<<<w.ntiles, kThreads, 0, s>>>(w);
+    k_mm_label<<<wide, kThreads, 0, s>>>(w);
+    ctx->launches += 2;
     int *h = (int *)ctx->h_pinned;
-    // acts (u64), then pending, sweeps, stop (int)
-    cudaMemcpyAsync(h, (const void *)Q.acts, sizeof(unsigned long long) + 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
-    cudaError_t e = ibip_sync(ctx, s);
+    cudaMemcpyAsync(h, w.ctr, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (ibip_sync(ctx, s) != cudaSuccess) return ibip_cuda_status(cudaGetLastError());
+    w.P = h[0];
+    int rounds = 0;
+    if (w.P > 0) {
+        // The tables share slots with the invasion, the EDT and the curve,
+        // none of which runs meanwhile.  No more than half the voxels are
+        // peaks; half an edge a voxel is usual.
+        int64_t cap = vox;
+        if (ctx->arena && ctx->slot[SC_LIST]) cap = std::min<int64_t>(cap, (int64_t)(ctx->slot_bytes[SC_LIST] / 4));
+        w.cap = (int)std::max<int64_t>(cap, 1);
+        w.node = (u64 *)ibip_scratch(ctx, SC_OKEY, ((size_t)w.P + 1) * sizeof(u64));
+        w.best = (u64 *)ibip_scratch(ctx, SC_HIST, ((size_t)w.P + 1) * sizeof(u64));
+        w.ea = (int *)ibip_scratch(ctx, SC_RANK, (size_t)w.cap * 4);
+        w.eb = (int *)ibip_scratch(ctx, SC_G2, (size_t)w.cap * 4);
+        w.ew = (int *)ibip_scratch(ctx, SC_LIST, (size_t)w.cap * 4);
+        if (!w.best || !w.node || !w.ea || !w.eb || !w.ew) return IBIP_ERR_OOM;
+    }
+    const int gp = (int)std::min<int64_t>(((int64_t)w.P + 1 + kThreads - 1) / kThreads, (int64_t)ctx->sm_count * 16);
+    if (w.P > 0) {
+        k_mm_nodes<<<gp, kThreads, 0, s>>>(w);
+        k_mm_pairs<false><<<wide, kThreads, 0, s>>>(w, 0);
+        k_mm_hook<<<gp, kThreads, 0, s>>>(w, 0);
+        k_mm_flatten<<<gp, kThreads, 0, s>>>(w, 0);
+        k_mm_pairs<true><<<std::min(wide, ctx->sm_count * 8), kThreads, 0, s>>>(w, 1);
+        ctx->launches += 5;
+        cudaMemcpyAsync(h, w.ctr, 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (ibip_sync(ctx, s) != cudaSuccess) return ibip_cuda_status(cudaGetLastError());
+        const bool list = h[1] <= w.cap;
+        bool more = h[1] > 0 && h[2] > 0;   // the list counts its unused entries too
+        if (list) w.listed = h[1];
+        const int ge = (int)std::min<int64_t>(((int64_t)h[1] + kThreads - 1) / kThreads + 1, (int64_t)ctx->sm_count * 16);
+        rounds = 1;
+        while (more) {
+            const int r1 = std::min(rounds + kRoundsPerSync, kMaxRoundsDev);
+            for (; rounds < r1; rounds++) {
+                if (list) k_mm_edges<<<ge, kThreads, 0, s>>>(w, rounds);
+                else k_mm_pairs<false><<<wide, kThreads, 0, s>>>(w, rounds);
+                k_mm_hook<<<gp, kThreads, 0, s>>>(w, rounds);
+                k_mm_flatten<<<gp, kThreads, 0, s>>>(w, rounds);
+                ctx->launches += 3;
+            }
+            cudaMemcpyAsync(h, w.ctr + 2 + rounds - 1, sizeof(int), cudaMemcpyDeviceToHost, s);
+            if (ibip_sync(ctx, s) != cudaSuccess) return ibip_cuda_status(cudaGetLastError());
+            more = h[0] > 0;
+            if (more && rounds == kMaxRoundsDev) {   // cannot happen: 2^63 basins
+                ibip_prof_end(ctx, IBIP_K_MAXIMIN);
+                return IBIP_ERR_NOT_CONVERGED;
+            }
+        }
+    }
+    k_mm_value<<<wide, kThreads, 0, s>>>(w);
+    ctx->launches++;
+    if (s != ctx->stream) {
+        // what follows on the slot's own stream
+        if (cudaEventRecord(ctx->ev_inv, s) != cudaSuccess ||
+            cudaStreamWaitEvent(ctx->stream, ctx->ev_inv, 0) != cudaSuccess)
+            return ibip_cuda_status(cudaGetLastError());
+    }
     ibip_prof_end(ctx, IBIP_K_MAXIMIN);
-    if (e != cudaSuccess) return ibip_cuda_status(e);
-    unsigned long long acts;
-    memcpy(&acts, h, sizeof(acts));
-    const int *c = h + 2;   // pending, sweeps, stop
-    ctx->inv_stats[30] = 0;   // no rounds
-    ctx->inv_stats[31] = (int64_t)acts;
-    ctx->inv_stats[32] = c[1];
-    return c[2] ? IBIP_ERR_NOT_CONVERGED : IBIP_OK;
+    ctx->inv_stats[30] = rounds;
+    ctx->inv_stats[31] = w.P;
+    ctx->inv_stats[32] = w.listed;
+    return ibip_cuda_status(cudaGetLastError());
 }
 
-// The round schedule as one ordinary launch per round, for contexts that
-// share the device with other streams: short launches let the blocks of
-// other streams' kernels (higher-priority ones first) in between rounds.
-int mm_run_round_launches(ibip_ctx *ctx, const MMArgs &a, int rounds)
+int ibip_maximin_multi(ibip_ctx *ctx, int n, const IbipMaximinJob *jobs)
 {
-    cudaStream_t s = ctx->stream;
-    int *h = (int *)ctx->h_pinned;
-    // rounds in chunks; the next round's list size is read back after
-    // each chunk (an empty round's launch returns at once).  A server
-    // slot issues them on its high-priority stream: each round is a
-    // short launch that would otherwise wait behind the wide kernels of
-    // the other jobs.
-    if (ctx->stream_inv) {
-        if (cudaEventRecord(ctx->ev_inv, s) != cudaSuccess ||
-            cudaStreamWaitEvent(ctx->stream_inv, ctx->ev_inv, 0) != cudaSuccess)
-            return ibip_cuda_status(cudaGetLastError());
-        s = ctx->stream_inv;
+    for (int j = 0; j < n;) {
+        int64_t vox = 0;
+        int m = j;
+        while (m < n && (m == j || vox + nvox(jobs[m].d) < (1ll << 31))) vox += nvox(jobs[m++].d);
+        const int st = mm_group(ctx, m - j, jobs + j);
+        if (st) return st;
+        j = m;
     }
-    constexpr int kChunkRounds = 16;
-    const int grid = ctx->sm_count;
-    int r = 0;
-    for (;;) {
-        for (int q = 0; q < kChunkRounds && r < rounds; q++, r++) {
-            k_mm_round<<<grid, kThreads, 0, s>>>(a, r);
-            IBIP_LAUNCH(ctx);
-        }
-        cudaMemcpyAsync(h, a.count + r, sizeof(int), cudaMemcpyDeviceToHost, s);
-        cudaError_t e = ibip_sync(ctx, s);
-        if (e != cudaSuccess) return ibip_cuda_status(e);
-        if (h[0] == 0) break;
-        if (r >= rounds) {
-            ibip_prof_end(ctx, IBIP_K_MAXIMIN);
-            return IBIP_ERR_NOT_CONVERGED;
-        }
-    }
-    ibip_prof_end(ctx, IBIP_K_MAXIMIN);
     return IBIP_OK;
 }
 
-// The round schedule: one cooperative grid (one large image), or one
-// launch per round in shared-device mode.
-int mm_run_rounds(ibip_ctx *ctx, int n, const std::vector<MMJob> &J, int nt, int rounds)
-{
-    cudaStream_t s = ctx->stream;
-    // layout: jobs | list0[nt] list1[nt] mark[nt] count[rounds+2] head[rounds+2] status[4]
-    const size_t jb = ((size_t)n * sizeof(MMJob) + 255) & ~(size_t)255;
-    const size_t ints = (size_t)3 * nt + 2 * ((size_t)rounds + 2) + 4;
-    char *w0 = (char *)ibip_scratch(ctx, SC_TILE, jb + ints * sizeof(int));
-    if (!w0) return IBIP_ERR_OOM;
-    MMJob *djobs = (MMJob *)w0;
-    int *w = (int *)(w0 + jb);
-    MMArgs a;
-    a.jobs = djobs; a.njobs = n;
-    a.list0 = w; a.list1 = w + nt; a.mark = w + 2 * nt;
-    a.count = w + 3 * nt; a.head = a.count + rounds + 2; a.status = a.head + rounds + 2;
-    a.max_rounds = rounds;
-    ibip_prof_begin(ctx, IBIP_K_MAXIMIN);
-    cudaMemcpyAsync(djobs, J.data(), (size_t)n * sizeof(MMJob), cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(a.mark, 0xff, (size_t)nt * sizeof(int), s);   // -1: never queued
-    cudaMemsetAsync(a.count, 0, (2 * ((size_t)rounds + 2) + 4) * sizeof(int), s);   // counts, heads, status
-    for (int j = 0; j < n; j++) {
-        k_mm_init<<<ctx->sm_count * 4, 256, 0, s>>>(J[j].val, J[j].nx, J[j].ny, J[j].nz, J[j].face, J[j].M);
-        IBIP_LAUNCH(ctx);
-    }
-    k_mm_seed<<<(nt + 255) / 256, 256, 0, s>>>(djobs, n, nt, a.list0, a.count, a.mark);
-    IBIP_LAUNCH(ctx);
-    if (ctx->no_coop) return mm_run_round_launches(ctx, a, rounds);
-    int *h = (int *)ctx->h_pinned;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mm_persistent, kThreads, 0) != cudaSuccess ||
-        per_sm < 1) {
-        cudaGetLastError();
-        return IBIP_ERR_CUDA;
-    }
-    int grid = ctx->sm_count * per_sm;
-    if (grid > nt) grid = nt;
-    void *args[] = {&a};
-    cudaError_t e = cudaLaunchCooperativeKernel((void *)k_mm_persistent, grid, kThreads, args, 0, s);
-    IBIP_LAUNCH(ctx);
-    if (e != cudaSuccess) return ibip_cuda_status(e);
-    cudaMemcpyAsync(h, a.status, 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
-    e = ibip_sync(ctx, s);
-    ibip_prof_end(ctx, IBIP_K_MAXIMIN);
-    if (e != cudaSuccess) return ibip_cuda_status(e);
-    // diagnostics of the last propagation: rounds, tile activations, sweeps
-    const int nr = h[0] < rounds ? h[0] : rounds, conv_flag = h[1], sweeps = h[2];
-    int *hc = (int *)ctx->h_pinned;
-    int64_t act = 0;
-    for (int r0 = 0; r0 < nr; r0 += 8192) {
-        const int c = nr - r0 < 8192 ? nr - r0 : 8192;
-        cudaMemcpyAsync(hc, a.count + r0, (size_t)c * sizeof(int), cudaMemcpyDeviceToHost, s);
-        if (ibip_sync(ctx, s) != cudaSuccess) return IBIP_ERR_CUDA;
-        for (int q = 0; q < c; q++) act += hc[q];
-    }
-    ctx->inv_stats[30] = nr;
-    ctx->inv_stats[31] = act;
-    ctx->inv_stats[32] = sweeps;
-    return conv_flag ? IBIP_ERR_NOT_CONVERGED : IBIP_OK;
-}
-
-}  // namespace
-
-int ibip_maximin_multi(ibip_ctx *ctx, int n, const IbipMaximinJob *jobs, int max_rounds)
-{
-    if (n <= 0) return IBIP_OK;
-    std::vector<MMJob> J(n);
-    int64_t ntot = 0;
-    for (int j = 0; j < n; j++) {
-        const ibip_dims d = jobs[j].d;
-        J[j].val = jobs[j].val; J[j].M = jobs[j].M;
-        J[j].nx = d.nx; J[j].ny = d.ny; J[j].nz = d.nz;
-        J[j].tx = (d.nx + TX - 1) / TX; J[j].ty = (d.ny + TY - 1) / TY; J[j].tz = (d.nz + TZ - 1) / TZ;
-        J[j].face = jobs[j].face;
-        J[j].tile0 = (int)ntot;
-        ntot += (int64_t)J[j].tx * J[j].ty * J[j].tz;
-    }
-    if (ntot >= (1ll << 30)) return IBIP_ERR_ARG;
-    const int nt = (int)ntot;
-    const int rounds = max_rounds < kMaxRoundsDev ? max_rounds : kMaxRoundsDev;
-    // beside other streams' kernels (shared-device mode): rounds as short
-    // launches; neither a cooperative grid, which needs every block
-    // resident, nor the queue, whose resident blocks would hold the SMs
-    // against other streams' kernels until the propagation ends
-    if (!ctx->no_coop && (n > 1 || nt < kQueueTiles)) return mm_run_queue(ctx, n, J, nt, rounds);
-    return mm_run_rounds(ctx, n, J, nt, rounds);
-}
-
-int ibip_maximin_launch(ibip_ctx *ctx, const int32_t *val, ibip_dims d, int face, int32_t *M, int max_rounds)
+int ibip_maximin_launch(ibip_ctx *ctx, const int32_t *val, ibip_dims d, int face, int32_t *M)
 {
     IbipMaximinJob j{val, d, face, M};
-    return ibip_maximin_multi(ctx, 1, &j, max_rounds);
+    return ibip_maximin_multi(ctx, 1, &j);
 }
