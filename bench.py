@@ -15,10 +15,10 @@ are bit-exact with the CPU oracle (tests/).
 value  = voxels per second through the whole path (device-resident inputs);
 e2e    = the same through the public API with the image copied from pinned
          host memory and seq_out + Pc curve copied back inside the timing;
-roofline = the dominant kernel class (the invasion: a latency-bound loop on
-         one CTA, whose figure of merit is its step latency), with
-         roofline.hbm_kernels giving every HBM-bound class (EDT, rank sort,
-         widest path, trapped mask, Pc, opening dilation) as algorithmic
+roofline = the dominant kernel class (the invasion: bound by its longest
+         chain of dependent steps, whose figure of merit is its step
+         latency), with roofline.hbm_kernels giving every HBM-bound class
+         (EDT, the invasion's statistics pass, widest path, trapped mask, Pc, opening dilation) as algorithmic
          bytes / live CUDA-event time / measured HBM copy bandwidth;
 cpu_baseline = the plain C oracle on this host's cores (rank 0, N=1), on a
          bounded sample when a full pass would take minutes.
@@ -59,20 +59,6 @@ CLASS_NAMES = ["edt", "rank", "invade", "maximin", "trap", "pc", "dilate"]
 NCU_TRAFFIC = {
     "edt": {"bytes_per_voxel": 15.699, "src": {"paper_2101_03240_gb300/csrc/edt.cu": "1dad9f25dc064510"},
              "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
-    "rank": {"bytes_per_voxel": 45.067, "src": {"paper_2101_03240_gb300/csrc/invade.cu": "0f50d49a6694434e", "paper_2101_03240_gb300/csrc/scan.cu": "7ae2dbb22ecb3ed4"},
-             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
-    "maximin": {"bytes_per_voxel": 300.551, "src": {"paper_2101_03240_gb300/csrc/maximin.cu": "2a905a8c9742daf6"},
-             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
-    "maximin_trim": {"bytes_per_voxel": 105.892, "src": {"paper_2101_03240_gb300/csrc/maximin.cu": "2a905a8c9742daf6"},
-             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
-    "trap": {"bytes_per_voxel": 12.615, "src": {"paper_2101_03240_gb300/csrc/pc.cu": "eb392979ed4ea0da"},
-             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
-    "pc": {"bytes_per_voxel": 4.631, "src": {"paper_2101_03240_gb300/csrc/pc.cu": "eb392979ed4ea0da", "paper_2101_03240_gb300/csrc/scan.cu": "7ae2dbb22ecb3ed4"},
-             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
-    "dilate": {"bytes_per_voxel": 14.721, "src": {"paper_2101_03240_gb300/csrc/edt.cu": "1dad9f25dc064510"},
-             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
-    "invade": {"bytes_per_voxel": 38.414, "src": {"paper_2101_03240_gb300/csrc/invade.cu": "0f50d49a6694434e"},
-               "workload": "blobs512", "capture": "profiles/k_invade_blobs512_traffic.md"},
 }
 
 
@@ -128,7 +114,7 @@ def parse():
                     help="serve: device arena of the server (20 GB: below the stream's peak demand, so admission binds)")
     ap.add_argument("--slots", type=int, default=16,
                     help="serve: worker slots (the stream keeps ~6 jobs in flight on average; 16 slots keep the "
-                         "jobs' kernels from crowding each other's one-CTA invasions)")
+                         "jobs' kernels from crowding each other's invasions)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--rule", choices=["frontier", "paper"], default="frontier",
                     help="invasion rule: the frontier rule, or Section 2.1 as printed (all ties, trunc radius)")
@@ -651,13 +637,11 @@ def run_ours(args, rank, world):
     cen = torch.empty(N, dtype=torch.int32, device=dev)
     dt2 = torch.empty(img_d.shape, dtype=torch.int32, device=dev)
 
-    # The opening needs only the image and dt2, not the invasion, whose one
-    # CTA leaves the other SMs idle for most of the step: it runs on a second
-    # context (shared-device mode: no cooperative grid beside the running
-    # invasion) on a low-priority stream, driven from a worker thread while
-    # this thread waits on the invasion; the rest of the path runs on a
-    # high-priority stream.  The opening is joined as soon as the invasion
-    # returns, so trapping's cooperative grid never starts beside it.
+    # The opening needs only the image and dt2, not the invasion: it runs on a
+    # second context (shared-device mode: no cooperative grid of its own) on a
+    # low-priority stream, driven from a worker thread while this thread waits
+    # on the invasion; the rest of the path runs on a high-priority stream.
+    # The opening is joined as soon as the invasion returns.
     from concurrent.futures import ThreadPoolExecutor
     ctx_open = ibip.Context(local)
     ctx_open.set_shared_device(True)
@@ -731,8 +715,8 @@ def run_ours(args, rank, world):
         (m0, n0), (m1, n1) = ctx.profile_read(c), ctx_open.profile_read(c)
         prof[CLASS_NAMES[c]] = (m0 + m1, n0 + n1)
         prof_open[CLASS_NAMES[c]] = (m1, n1)
-    # the widest path runs twice: trapping on the critical path (one
-    # cooperative grid) and the opening's trim beside the invasion
+    # the widest path runs twice: trapping on the critical path and the
+    # opening's trim beside the invasion
     mm_trap = (prof["maximin"][0] - prof_open["maximin"][0], prof["maximin"][1] - prof_open["maximin"][1])
     ctx.profile(False)
     ctx_open.profile(False)
@@ -847,11 +831,11 @@ def run_ours(args, rank, world):
     alg = {
         "edt": 5 * N,                                   # read image, write dt2
         "invade": 8 * N + 8 * K,                        # read dt2, write seq, r2+centre per step
-        "rank": 4 * N + 4 * N + 8 * npore,              # read dt2, write rank, write (idx, dt2) by rank
+        "rank": 4 * N,                                  # read dt2 (largest value, pore count)
         "maximin": 8 * N,                               # read values, write widest-path field
         "trap": 4 * N + 4 * N + 1 * N + 4 * N,          # read seq, M; write mask, seq_out
         "pc": 4 * N + 12 * K,                           # histogram of seq; S, Pc, r2 per step
-        "dilate": (4 + 4 + 4) * N,                      # per level: read W, read/write level
+        "dilate": (4 + 4 + 4) * N,                      # up to 32 levels: read W, read/write level
     }
     kinfo = {}
     for c, (tms, spans) in prof.items():
@@ -875,18 +859,17 @@ def run_ours(args, rank, world):
                           "frac": ach / hbm_peak, "traffic": traffic_per_launch(c, N, w.name),
                           "algorithmic_bytes_per_launch": int(alg[c]),
                           "ms_per_launch": per, "launches_per_step": spans // max(args.steps, 1)}
-    hbm_kernels["maximin"]["note"] = "trapping's widest path: one cooperative grid on the critical path"
+    hbm_kernels["maximin"]["note"] = "trapping's widest path, on the critical path"
     if "maximin_trim" in hbm_kernels:
-        hbm_kernels["maximin_trim"]["note"] = ("the opening's trim: the same propagation in shared-device mode "
-                                               "(one launch per round), overlapped with the invasion")
+        hbm_kernels["maximin_trim"]["note"] = "the opening's trim: the same kernels beside the invasion"
     per_launch = prof[dom][0] / max(prof[dom][1], 1)
     achieved = alg[dom] / (per_launch * 1e-3) / 1e9
     roofline = {"bound": "hbm", "kernel": dom, "achieved": round(achieved, 3), "peak": hbm_peak,
                 "unit": "GB/s", "frac": achieved / hbm_peak, "traffic": traffic_per_launch(dom, N, w.name),
                 "peak_source": "measured" if pk else "fallback",
-                "note": "the invasion is a serial, latency-bound loop on one CTA: achieved counts its "
+                "note": "the invasion is bound by its longest chain of dependent steps: achieved counts its "
                         "algorithmic bytes (dt2 read + seq write + step arrays), traffic is ncu's DRAM bytes per "
-                        "launch (lines re-read between overlapping balls); its figure of merit is the step "
+                        "launch where captured; its figure of merit is the step "
                         "latency (invasion_step_times, invasion_us_per_step); hbm_kernels holds the HBM-bound "
                         "classes against the measured copy bandwidth",
                 "hbm_kernels": hbm_kernels}
