@@ -693,22 +693,33 @@ int ibip_morph_drainage_ex(ibip_ctx *ctx, const uint8_t *image, const int32_t *d
     if (st) return st;
     int first = 0;
     while (first < n_levels && h_r2_levels[first] > wmax) first++;
-    if (n_levels <= 254) {
-        uint8_t *fl = (uint8_t *)ibip_scratch(ctx, SC_FL, (size_t)nvox(dims) + 256 * sizeof(int32_t) + 256);
-        if (!fl) return IBIP_ERR_OOM;
-        int32_t *T_dev = (int32_t *)(fl + (((size_t)nvox(dims) + 255) & ~(size_t)255));
-        cudaMemcpyAsync(T_dev, h_r2_levels, (size_t)n_levels * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream);
-        st = ibip_first_level_launch(ctx, W, dims, T_dev, n_levels, fl);
+    // a level goes by bit planes where those take it, else by EDT passes: from
+    // a byte per voxel (its first level) for up to 254 levels, else from W
+    uint8_t *fl = nullptr;
+    for (int i = first; i < n_levels;) {
+        int next = i;
+        st = ibip_open_run(ctx, W, dims, h_r2_levels, Td, i, n_levels, level, &next);
         if (st) return st;
-        for (int i = first; i < n_levels; i++) {
-            st = ibip_dilate_first_level_launch(ctx, fl, Td[i], i, dims, level);
-            if (st) return st;
+        if (next > i) {
+            i = next;
+            continue;
         }
-    } else {
-        for (int i = first; i < n_levels; i++) {
+        if (n_levels > 254) {
             st = ibip_dilate_level_launch(ctx, W, h_r2_levels[i], Td[i], i + 1, dims, level);
-            if (st) return st;
+        } else {
+            if (!fl) {
+                fl = (uint8_t *)ibip_scratch(ctx, SC_FL, (size_t)nvox(dims) + 256 * sizeof(int32_t) + 256);
+                if (!fl) return IBIP_ERR_OOM;
+                int32_t *T_dev = (int32_t *)(fl + (((size_t)nvox(dims) + 255) & ~(size_t)255));
+                cudaMemcpyAsync(T_dev, h_r2_levels, (size_t)n_levels * sizeof(int32_t), cudaMemcpyHostToDevice,
+                                ctx->stream);
+                st = ibip_first_level_launch(ctx, W, dims, T_dev, n_levels, fl);
+                if (st) return st;
+            }
+            st = ibip_dilate_first_level_launch(ctx, fl, Td[i], i, dims, level);
         }
+        if (st) return st;
+        i++;
     }
     return ibip_level_counts(ctx, level, dims, n_levels, h_counts);
 }

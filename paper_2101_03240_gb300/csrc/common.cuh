@@ -167,6 +167,10 @@ int ibip_dilate_level_launch(ibip_ctx *ctx, const int32_t *W, int32_t T, int32_t
 int ibip_first_level_launch(ibip_ctx *ctx, const int32_t *W, ibip_dims d, const int32_t *T_dev, int L, uint8_t *fl);
 int ibip_dilate_first_level_launch(ibip_ctx *ctx, const uint8_t *fl, int32_t T, int32_t i, ibip_dims d,
                                    int32_t *level);
+// MIO on bit planes: levels [i, *next) where the kernel takes them (*next == i
+// where it does not take level i).
+int ibip_open_run(ibip_ctx *ctx, const int32_t *W, ibip_dims d, const int32_t *T, const int32_t *Td, int i, int n,
+                  int32_t *level, int *next);
 int ibip_max_launch(ibip_ctx *ctx, const int32_t *a, int64_t n, int *h_max);
 // Maximin propagation from a face through voxels with val != 0 (val == -1
 // counts as +inf).  Writes M (-1 where unreachable).
