@@ -786,7 +786,7 @@ int ibip_invade_batched(ibip_ctx *ctx, int32_t n, ibip_job *jobs)
     P.M = mm_total ? (int32_t *)ibip_scratch(ctx, SC_MM, (size_t)mm_total * sizeof(int32_t)) : nullptr;
     // the widest path's tables: basins are a few percent of the voxels
     const size_t basins = (size_t)mm_total / 8 + 1024;
-    if ((mm_total && (!P.M || !ibip_scratch(ctx, SC_TILE, (size_t)n * 128 + 1024) ||
+    if ((mm_total && (!P.M || !ibip_scratch(ctx, SC_TILE, ibip_maximin_table_bytes(ctx, n, mm_total)) ||
                       !ibip_scratch(ctx, SC_OKEY, basins * 8) || !ibip_scratch(ctx, SC_HIST, basins * 8) ||
                       !ibip_scratch(ctx, SC_RANK, (size_t)mm_total * 4) ||
                       !ibip_scratch(ctx, SC_G2, (size_t)mm_total * 4) ||
