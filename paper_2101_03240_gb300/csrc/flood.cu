@@ -354,6 +354,9 @@ enum Team { WARP, BLOCK, LONG };   // a group on a warp, on the CTA, on the CTA 
 // queue.  What bounds a step is the chain of instructions and round trips
 // from one step to the next, not the work: rows are dealt to the warps in
 // turn, so that the full rows at the centre are spread over all of them.
+// Neither the state image nor the planes change while groups run, so their
+// loads go through the L1 (the barrier before the round orders them): 512^3
+// blobs 105.5 -> 102.5 ms, 200^3 pack 19.0 -> 18.4.
 // A long group takes its masks from two bit planes (`fresh`: uninvaded, no
 // candidate; `root_bits`: the phase's roots), two words for a row instead of
 // up to four 16-byte chunks of the state image.
@@ -507,10 +510,10 @@ __device__ __noinline__ LogPos run_group(const Flood &f, const Phase &ph_in, Sha
                             const bool two = (z0 >> 5) != (z1 >> 5);
                             u32 f0 = 0, f1 = 0, g0 = 0, g1 = 0;
                             if (in_range(ctl, w, nx * ny * NW, P_PLANE) && in_range(ctl, w + two, nx * ny * NW, P_PLANE)) {
-                                f0 = __ldcg(fresh + w);
-                                g0 = __ldcg(root_bits + w);
-                                f1 = __ldcg(fresh + w + two);
-                                g1 = __ldcg(root_bits + w + two);
+                                f0 = fresh[w];
+                                g0 = root_bits[w];
+                                f1 = fresh[w + two];
+                                g1 = root_bits[w + two];
                             }
                             const u32 span = 0xffffffffu >> (31 - (z1 - z0));
                             const u32 fr = __funnelshift_r(f0, f1, z0 & 31) & span;
@@ -529,7 +532,7 @@ __device__ __noinline__ LogPos run_group(const Flood &f, const Phase &ph_in, Sha
                         uint4 cw[kU];
 #pragma unroll
                         for (int u = 0; u < kU; u++)
-                            cw[u] = u < n_ch && in_range(ctl, c + u, (n_vox + 7) / 8, P_STATE) ? __ldcg(state + c + u)
+                            cw[u] = u < n_ch && in_range(ctl, c + u, (n_vox + 7) / 8, P_STATE) ? state[c + u]
                                                                                              : make_uint4(0, 0, 0, 0);
 #pragma unroll
                         for (int u = 0; u < kU; u++) {
@@ -579,7 +582,7 @@ __device__ __noinline__ LogPos run_group(const Flood &f, const Phase &ph_in, Sha
                             const int u = (vx * ny + vy) * nz + vz;
                             if (in_range(ctl, u, n_vox, P_CLAIM)) {
                                 old = atomicMax(claim + u, gid);
-                                if (!inside) val = (int)__ldcg((const unsigned short *)state + u);   // beside the claim
+                                if (!inside) val = (int)((const unsigned short *)state)[u];   // beside the claim
                             }
                         }
                         bool push = old != gid;
