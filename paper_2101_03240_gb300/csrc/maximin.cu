@@ -219,76 +219,102 @@ constexpr int kBlockEdges = 512;
 // list, of each run of lanes with the same two roots only the largest; else
 // they are offered to the two roots (the outside, root P, takes none).
 template <bool LIST>
-__global__ void __launch_bounds__(kThreads) k_mm_pairs(MMWork w, int round)
+__global__ void __launch_bounds__(kThreads, 8) k_mm_pairs(MMWork w, int round)
 {
     if (round > 0 && __ldcg(w.ctr + 2 + round - 1) == 0) return;
     const int lane = threadIdx.x & 31;
     int lbase = 0, lleft = 0;   // list entries of the warp
+    bool full = false;          // the list has run out
+    const bool first = round == 0;
     for_segments(w, [&](const MMJob &J, int x, int y, int z, int64_t v, bool in) {
+        // the loads of all four directions side by side: labels, then values
+        // and roots, then the roots' best edges
+        const int64_t off[3] = {1, J.nz, (int64_t)J.ny * J.nz};
+        const bool ok[3] = {z < J.nz - 1, y < J.ny - 1, x < J.nx - 1};
         const uint32_t lb = in ? __ldcg(J.M + v) : kBlocked;
+        uint32_t lu[3];
+#pragma unroll
+        for (int d = 0; d < 3; d++) lu[d] = in && ok[d] ? __ldcg(J.M + v + off[d]) : kBlocked;
         const int val = lb != kBlocked ? as_val(__ldg(J.val + v)) : 0;
         uint32_t a = lb == kBlocked ? kBlocked : lb & ~kPeak;
-        const bool first = round == 0;
+        uint32_t bs[4];
+        int ws[4];
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            bs[d] = kBlocked;
+            ws[d] = 0;
+            if (lb != kBlocked && lu[d] != kBlocked && lu[d] != lb) {
+                bs[d] = lu[d] & ~kPeak;
+                ws[d] = as_val(__ldg(J.val + v + off[d]));
+                if (!first) bs[d] = parent_of(w, bs[d]);
+            }
+        }
         if (!first && a != kBlocked) a = parent_of(w, a);
 #pragma unroll
-        for (int d = 0; d < 4; d++) {
-            uint32_t b = kBlocked;
-            int wt = 0;
-            if (a != kBlocked) {
-                if (d < 3) {
-                    const bool ok = d == 0 ? z < J.nz - 1 : d == 1 ? y < J.ny - 1 : x < J.nx - 1;
-                    const int64_t u = v + (d == 0 ? 1 : d == 1 ? (int64_t)J.nz : (int64_t)J.ny * J.nz);
-                    if (ok) {
-                        const uint32_t lu = __ldcg(J.M + u);
-                        if (lu != kBlocked && lu != lb) {
-                            b = lu & ~kPeak;
-                            if (!first) b = parent_of(w, b);
-                            wt = min(val, as_val(__ldg(J.val + u)));
-                        }
-                    }
-                } else if (d_on_face(x, y, z, J.nx, J.ny, J.nz, J.face)) {
-                    b = (uint32_t)w.P;
-                    wt = val;
-                }
-            }
-            bool edge = b != kBlocked && a != b;
-            if (LIST) {
-                if (!__any_sync(0xffffffffu, edge)) continue;
-                // runs of the same two roots: the largest weight, kept by the
-                // last lane of the run
-                const uint32_t pa = __shfl_up_sync(0xffffffffu, a, 1), pb = __shfl_up_sync(0xffffffffu, b, 1);
-                const bool cont = __shfl_up_sync(0xffffffffu, (int)edge, 1) && lane > 0 && edge && pa == a && pb == b;
-                const unsigned heads = __ballot_sync(0xffffffffu, !cont);
-                const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+        for (int d = 0; d < 3; d++) ws[d] = min(ws[d], val);
+        const bool face = a != kBlocked && d_on_face(x, y, z, J.nx, J.ny, J.nz, J.face);
+        bs[3] = face ? (uint32_t)w.P : kBlocked;
+        ws[3] = val;
+        if (!LIST) {
+            u64 top = 0, had_b[3], had_a = 0;
+            bool any = face && a != (uint32_t)w.P;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int t = __shfl_up_sync(0xffffffffu, wt, o);
-                    if (lane - o >= start) wt = max(wt, t);
-                }
-                edge = edge && (lane == 31 || ((heads >> (lane + 1)) & 1u));
-                const unsigned m = __ballot_sync(0xffffffffu, edge);
-                const int need = __popc(m), k = __popc(m & ((1u << lane) - 1));
-                int pos = lbase + k;
-                if (lleft < need) {
-                    int nb = 0;
-                    if (lane == 0) nb = atomicAdd(w.ctr + 1, kChunk);
-                    nb = __shfl_sync(0xffffffffu, nb, 0) - lleft;
-                    if (k >= lleft) pos = nb + k;
-                    lbase = nb;
-                    lleft += kChunk;
-                }
-                if (edge && pos < w.cap) {
-                    w.ea[pos] = (int)a;
-                    w.eb[pos] = (int)b;
-                    w.ew[pos] = wt;
-                }
-                lbase += need;
-                lleft -= need;
-            } else if (edge) {
-                const u64 key = (u64)(uint32_t)wt << 33 | (u64)(4 * (J.vox0 + v) + d);
-                if (a != (uint32_t)w.P) offer(w, a, key);
-                if (b != (uint32_t)w.P) offer(w, b, key);
+            for (int d = 0; d < 3; d++) {
+                had_b[d] = ~0ull;
+                if (bs[d] == kBlocked || bs[d] == a) continue;
+                any = true;
+                if (bs[d] != (uint32_t)w.P) had_b[d] = __ldcg(w.best + bs[d]);
             }
+            if (!any) return;
+            if (a != (uint32_t)w.P) had_a = __ldcg(w.best + a);
+#pragma unroll
+            for (int d = 0; d < 4; d++) {
+                if (bs[d] == kBlocked || bs[d] == a) continue;
+                const u64 key = (u64)(uint32_t)ws[d] << 33 | (u64)(4 * (J.vox0 + v) + d);
+                top = key > top ? key : top;
+                if (d < 3 && key > had_b[d]) atomicMax(w.best + bs[d], key);
+            }
+            if (a != (uint32_t)w.P && top > had_a) atomicMax(w.best + a, top);
+            return;
+        }
+#pragma unroll
+        for (int d = 0; d < 4; d++) {
+            const uint32_t b = bs[d];
+            int wt = ws[d];
+            bool edge = b != kBlocked && a != b;
+            if (!__any_sync(0xffffffffu, edge)) continue;
+            // runs of the same two roots: the largest weight, kept by the
+            // last lane of the run
+            const uint32_t pa = __shfl_up_sync(0xffffffffu, a, 1), pb = __shfl_up_sync(0xffffffffu, b, 1);
+            const bool cont = __shfl_up_sync(0xffffffffu, (int)edge, 1) && lane > 0 && edge && pa == a && pb == b;
+            const unsigned heads = __ballot_sync(0xffffffffu, !cont);
+            const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, wt, o);
+                if (lane - o >= start) wt = max(wt, t);
+            }
+            edge = edge && (lane == 31 || ((heads >> (lane + 1)) & 1u));
+            const unsigned m = __ballot_sync(0xffffffffu, edge);
+            const int need = __popc(m), k = __popc(m & ((1u << lane) - 1));
+            int pos = lbase + k;
+            if (lleft < need) {
+                int nb = w.cap;
+                if (lane == 0 && !full) nb = atomicAdd(w.ctr + 1, kChunk);
+                nb = __shfl_sync(0xffffffffu, nb, 0);
+                full = nb >= w.cap;   // the counter is left alone then (pairs may number three a voxel)
+                nb -= lleft;
+                if (k >= lleft) pos = nb + k;
+                lbase = nb;
+                lleft += kChunk;
+            }
+            if (edge && pos < w.cap) {
+                w.ea[pos] = (int)a;
+                w.eb[pos] = (int)b;
+                w.ew[pos] = wt;
+            }
+            lbase += need;
+            lleft -= need;
         }
     });
     if (LIST)   // the entries left over are no edges
@@ -428,10 +454,11 @@ __global__ void __launch_bounds__(kThreads) k_mm_value(MMWork w)
     for_segments(w, [&](const MMJob &J, int, int, int, int64_t v, bool in) {
         if (!in) return;
         const uint32_t lb = __ldcg(J.M + v);
+        const int val = as_val(__ldg(J.val + v));
         int m = -1;
         if (lb != kBlocked) {
             const u64 x = __ldcg(w.node + (lb & ~kPeak));
-            if ((uint32_t)x == (uint32_t)w.P) m = min(as_val(__ldg(J.val + v)), (int)(x >> 32));
+            if ((uint32_t)x == (uint32_t)w.P) m = min(val, (int)(x >> 32));
         }
         J.M[v] = (uint32_t)m;
     });
@@ -506,7 +533,7 @@ static int mm_group(ibip_ctx *ctx, int n, const IbipMaximinJob *jobs)
         // peaks; half an edge a voxel is usual.
         int64_t cap = vox;
         if (ctx->arena && ctx->slot[SC_LIST]) cap = std::min<int64_t>(cap, (int64_t)(ctx->slot_bytes[SC_LIST] / 4));
-        w.cap = (int)std::max<int64_t>(cap, 1);
+        w.cap = (int)std::min<int64_t>(std::max<int64_t>(cap, 1), 1 << 30);   // places stay below 2^31
         w.node = (u64 *)ibip_scratch(ctx, SC_OKEY, ((size_t)w.P + 1) * sizeof(u64));
         w.best = (u64 *)ibip_scratch(ctx, SC_HIST, ((size_t)w.P + 1) * sizeof(u64));
         w.ea = (int *)ibip_scratch(ctx, SC_RANK, (size_t)w.cap * 4);
