@@ -55,7 +55,7 @@ typedef enum {
     IBIP_ERR_CUDA = -2,          /* a CUDA runtime call failed */
     IBIP_ERR_OOM = -3,           /* scratch allocation failed */
     IBIP_ERR_STEP_LIMIT = -4,    /* invasion stopped at max_steps with candidates left */
-    IBIP_ERR_NOT_CONVERGED = -5, /* propagation hit its round or activation limit, or stalled */
+    IBIP_ERR_NOT_CONVERGED = -5, /* a device loop hit its round or step limit, or stalled */
     IBIP_ERR_CANCELLED = -6,     /* the invasion stopped at a cancel request (ibip_cancel) */
     IBIP_ERR_BOUNDS = -7,        /* a device-side index check failed (progress guard; any
                                     index of the invasion loop in a build with IBIP_CHECKED) */
@@ -96,14 +96,11 @@ IBIP_API int ibip_get_stream(const ibip_ctx *ctx, void **h_stream);
 /* Whether this context's kernels may run beside long-running kernels of
  * other streams or contexts on the same device (on != 0), for instance an
  * invasion running on another stream while this context computes the
- * opening.  The widest-path propagation (trapping, the opening's trim) then
- * runs one ordinary launch per round, the host reading the next round's
- * list size every 16 rounds, so that the other streams' blocks get in
- * between rounds.  It never runs as one cooperative grid, whose blocks must
- * all be resident at once, nor on its work queue, whose resident blocks
- * would hold the SMs until the propagation ends; those serve a context
- * that has the device to itself.  Results are the same every way.  Default
- * off; server slots always run this way.  IBIP_ERR_ARG for a NULL ctx. */
+ * opening.  An invasion then runs on one thread-block cluster whatever the
+ * image's size, never as a cooperative grid, whose blocks must all be
+ * resident at once; every other kernel is an ordinary launch either way.
+ * Results are the same both ways.  Default off; server slots always run
+ * this way.  IBIP_ERR_ARG for a NULL ctx. */
 IBIP_API int ibip_set_shared_device(ibip_ctx *ctx, int on);
 
 /* Squared Euclidean distance transform of the pore space (Section 2.1,
@@ -216,8 +213,8 @@ IBIP_API int ibip_invade_literal(ibip_ctx *ctx, const uint8_t *image, const int3
  *             1..K' in order (Section 2.2.3, contiguous sequence).
  *   trapped:  uint8[N] output, 1 = trapped.
  *   seq_out:  int32[N] output (seq with trapped voxels set to -1), or NULL.
- * Synchronous (the propagation loop checks convergence on the host);
- * returns IBIP_ERR_NOT_CONVERGED if the round limit was reached. */
+ * Synchronous (the host counts the rounds of the widest-path forest);
+ * returns IBIP_ERR_NOT_CONVERGED if their limit was reached. */
 IBIP_API int ibip_trapping(ibip_ctx *ctx, const int32_t *seq, ibip_dims dims, int outlet, int rerank,
                   uint8_t *trapped, int32_t *seq_out);
 
@@ -349,8 +346,8 @@ typedef struct {
  * (Section 2.1), trapping (Section 2.2.3) when `trapped` is given, and the
  * saturation / Pc curve (Sections 2.2.1-2.2.2; computed from seq_out when
  * trapping ran, else from seq) when `sat_per_step` is given.  The
- * invasions of all images run in one launch, one persistent CTA per image,
- * largest first; results equal the per-image calls bit for bit.
+ * invasions of all images run in one launch, one thread-block cluster per
+ * image, largest first; results equal the per-image calls bit for bit.
  *   h_jobs: host array of n jobs (1 <= n <= 4096); n_steps and status are
  *           written back.  An image's pore count must stay below 2^25,
  *           the whole batch's below 2^31.
@@ -428,8 +425,8 @@ IBIP_API int64_t ibip_job_footprint(ibip_dims dims, int with_dt2);
 /* Creates a server on ctx's device (ctx itself is not used afterwards).
  * 1 <= max_slots <= 128.  Allocates the arena (IBIP_ERR_OOM if it cannot).
  * Each slot has two streams: its wide kernels (EDT, rank sort, curve) at
- * the device's lowest stream priority, its one-CTA invasion and the
- * per-round widest-path launches at the highest; its waits sleep on
+ * the device's lowest stream priority, its invasion (one cluster) and the
+ * widest-path launches at the highest; its waits sleep on
  * blocking-sync events.  CUDA maps streams onto CUDA_DEVICE_MAX_CONNECTIONS
  * hardware queues (8 by default): with more streams than queues a long
  * invasion kernel holds up the later launches of every stream sharing its
@@ -521,8 +518,8 @@ IBIP_API int64_t ibip_launch_count(const ibip_ctx *ctx);
 typedef enum {
     IBIP_K_EDT = 0,       /* the three EDT passes of ibip_edt / ibip_invade */
     IBIP_K_RANK = 1,      /* rank sort and bit-plane setup of ibip_invade */
-    IBIP_K_INVADE = 2,    /* the persistent invasion kernel */
-    IBIP_K_MAXIMIN = 3,   /* widest-path propagation rounds (trapping, opening) */
+    IBIP_K_INVADE = 2,    /* the invasion kernel */
+    IBIP_K_MAXIMIN = 3,   /* widest path (trapping, opening) */
     IBIP_K_TRAP = 4,      /* trapped mask, seq_out and re-ranking */
     IBIP_K_PC = 5,        /* histogram, scan, saturation and Pc */
     IBIP_K_DILATE = 6,    /* per-level dilation passes of the opening */
@@ -544,8 +541,12 @@ IBIP_API int ibip_profile_read(ibip_ctx *ctx, int cls, double *h_ms, int64_t *h_
  * CTA).  The cycle entries are measured only by calls made while a trace is
  * set (ibip_invade_trace), which run a separate, timed build of the loop;
  * otherwise they read 0 (the clock reads would cost the loop about a tenth
- * of its time).  Writes up to n (at most 48) of:
- *   0 steps, 1 status, 2 iterations of the main loop,
+ * of its time).  A call that ran by value phases (untraced calls, but for
+ * images without solid or with values above 32767) reports entries 0-2 and
+ * 30-34; the others describe the one-CTA loop.  Writes up to n (at most 48)
+ * of:
+ *   0 steps, 1 status, 2 iterations of the main loop (by phases: rounds of
+ *   groups),
  *   3-5 cycles selecting, bounding (candidate shell) and committing,
  *   6 batch items taken, 7 batch items committed, 8 stale summary bits
  *   cleared, 9 ball rows committed,
@@ -557,10 +558,8 @@ IBIP_API int ibip_profile_read(ibip_ctx *ctx, int cls, double *h_ms, int64_t *h_
  *   24-25 bound stages 1 (shell listing) and 2 (rank lookups),
  *   26-27 commit stage 1 (stamping) and the rest (queueing),
  *   28-29 and 33 the single-voxel loop's gather, bound and commit cycles,
- *   30-32 rounds (0 on the work queue, none counted in per-round
- *   launches), tile activations and relaxation
- *   sweeps of the context's last widest-path propagation (trapping or the
- *   opening's trim),
+ *   30-32 rounds, basins and listed edges (-1: too many to list) of the
+ *   context's last widest-path forest (trapping or the opening's trim),
  *   34 out-of-range accesses counted by a checked build (IBIP_CHECKED),
  *   35 rank of the first voxel with the smallest dt2,
  *   36 batches seen by the trace (ibip_invade_trace; counted beyond its
@@ -613,8 +612,9 @@ IBIP_API int ibip_edt_tiles(ibip_ctx *ctx, ibip_dims dims, int *h_z_warps, int *
  * it starts; on = 0 withdraws the request.  Safe to call from another host
  * thread while ibip_invade / ibip_invade_ex / ibip_invade_batched block.
  * The flag lives in host-mapped memory; the invasion kernel reads it every
- * 16 batches of its main loop and every 64 of its single-voxel loop, and
- * stops before committing the next batch: the call returns
+ * 4 value phases (the one-CTA loop every 16 batches of its main loop and
+ * every 64 of its single-voxel loop) and stops before the next phase or
+ * batch: the call returns
  * IBIP_ERR_CANCELLED with *h_n_steps = k, and seq, step_r2 and step_centre
  * hold a valid invasion of k steps, which ibip_invade_ex(resume = 1)
  * continues to the same result as an uninterrupted call.  Serving the

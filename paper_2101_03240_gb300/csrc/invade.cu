@@ -5,7 +5,12 @@
 // |p - c|^2 < dt2[c].  Candidates are uninvaded pore voxels 6-adjacent to an
 // invaded voxel or lying on the inlet face.
 //
-// GPU design (one persistent CTA per image):
+// An invasion runs by value phases (flood.cu) on the whole GPU or on one
+// thread-block cluster, a batch on one cluster per image; set-up, launch and
+// completion are here.  Traced runs, images without solid, values above
+// 32767 and runs the phases give up take the loop below.
+//
+// The one-CTA loop:
 //  * Rank: pore voxels are ranked once by (dt2 descending, index ascending),
 //    a stable counting sort over dt2 values (per-chunk bucket counts, one
 //    flat scan, per-chunk stable scatter).  The priority order of the whole
@@ -39,7 +44,7 @@
 namespace {
 
 constexpr int kM = 64;           // batch size (items per iteration)
-constexpr int kNT = 768;         // threads of the persistent CTA (measured: 384, 512, 640, 768, 896, 1024 -> 1742, 1626, 1517, 1493, 1509, 1564 ms on the 512^3 blobs)
+constexpr int kNT = 768;         // threads of the loop's CTA (measured: 384, 512, 640, 768, 896, 1024 -> 1742, 1626, 1517, 1493, 1509, 1564 ms on the 512^3 blobs)
 constexpr int kChunk = 4096;     // voxels per rank-sort chunk (minimum)
 constexpr int kSmemL1Max = 12288;   // level-1 words of one image of a batched call (shared memory)
 constexpr int kNOut = kInvStats;   // int64 outputs of the invasion kernel

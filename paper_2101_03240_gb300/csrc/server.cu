@@ -14,12 +14,10 @@
 //     idle and the head job's piece can be carved, the head is admitted.  No
 //     job overtakes an earlier one, and a job that fits the arena is always
 //     admitted once the jobs ahead of it have run.
-//   - The invasion of a job is one persistent CTA, so the jobs in flight run
-//     side by side on different SMs; their EDT, rank, trapping and curve
-//     kernels interleave on the other streams.  Trapping uses the per-round
-//     launches of the widest-path propagation, never a cooperative grid,
-//     whose residency could not be guaranteed beside other streams' kernels,
-//     nor its work queue, whose resident blocks would hold the SMs.
+//   - The invasion of a job is one cluster of CTAs, so the jobs in flight run
+//     side by side on different SMs; their EDT, trapping and curve kernels
+//     interleave on the other streams.  No job starts a cooperative grid,
+//     whose residency could not be guaranteed beside other streams' kernels.
 #include <chrono>
 #include <condition_variable>
 #include <deque>

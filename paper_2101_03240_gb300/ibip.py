@@ -14,7 +14,7 @@ import threading
 
 # CUDA maps streams onto CUDA_DEVICE_MAX_CONNECTIONS hardware work queues
 # (8 unless set).  A server runs many slots, each with two streams; when
-# they outnumber the queues, a slot's long one-CTA invasion kernel holds up
+# they outnumber the queues, a slot's long invasion kernel holds up
 # every later launch of the other streams sharing its queue (small requests
 # then wait for seconds behind a large one).  32 is the largest value; it
 # only takes effect if set before the process creates its CUDA context, and
@@ -414,9 +414,8 @@ class Context:
 
     def set_shared_device(self, on: bool):
         """Let this context's kernels run beside long-running kernels of
-        other streams (ibip_set_shared_device): the widest-path propagation
-        then runs one ordinary launch per round instead of a cooperative
-        grid."""
+        other streams (ibip_set_shared_device): an invasion then runs on one
+        cluster instead of a cooperative grid."""
         st = _lib().ibip_set_shared_device(self._h, int(bool(on)))
         if st != OK:
             raise IbipError("ibip_set_shared_device", st)
