@@ -57,8 +57,6 @@ CLASS_NAMES = ["edt", "rank", "invade", "maximin", "trap", "pc", "dilate"]
 # digits of their SHA-256: when one has changed since, or the line runs
 # another workload, the class reports traffic null.
 NCU_TRAFFIC = {
-    "edt": {"bytes_per_voxel": 15.699, "src": {"paper_2101_03240_gb300/csrc/edt.cu": "1dad9f25dc064510"},
-             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
 }
 
 
