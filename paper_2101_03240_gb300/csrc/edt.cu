@@ -537,7 +537,7 @@ constexpr size_t kSmemBudget = 200 * 1024;
 template <class... P, class... A>
 void launch_pass(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
 {
-    if (smem > 48 * 1024)   // above what a kernel may use without asking
+    if (smem > 32 * 1024)   // with the static part at most 48 KB need no asking
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
     cudaLaunchAttribute behind{};
     behind.id = cudaLaunchAttributeProgrammaticStreamSerialization;
