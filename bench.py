@@ -57,6 +57,14 @@ CLASS_NAMES = ["edt", "rank", "invade", "maximin", "trap", "pc", "dilate"]
 # digits of their SHA-256: when one has changed since, or the line runs
 # another workload, the class reports traffic null.
 NCU_TRAFFIC = {
+    "maximin": {"bytes_per_voxel": 94.3, "src": {"paper_2101_03240_gb300/csrc/maximin.cu": "ca0532e531d61ed3"},
+             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
+    "trap": {"bytes_per_voxel": 12.61, "src": {"paper_2101_03240_gb300/csrc/pc.cu": "2033b9b8d7223d11"},
+             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
+    "pc": {"bytes_per_voxel": 4.77, "src": {"paper_2101_03240_gb300/csrc/pc.cu": "2033b9b8d7223d11", "paper_2101_03240_gb300/csrc/scan.cu": "7ae2dbb22ecb3ed4"},
+             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
+    "dilate": {"bytes_per_voxel": 19.11, "src": {"paper_2101_03240_gb300/csrc/opening.cu": "078490402b734dc2"},
+             "workload": "blobs512", "capture": "profiles/traffic_blobs512.md"},
 }
 
 
@@ -323,7 +331,7 @@ def run_batch(args, rank, world):
         "roofline": {"bound": "hbm", "kernel": "invade (batched)", "achieved": round(achieved, 3), "peak": hbm_peak,
                      "unit": "GB/s", "frac": achieved / hbm_peak, "traffic": None,
                      "peak_source": "measured" if pk else "fallback",
-                     "note": "one latency-bound CTA per image; bytes are the algorithmic minimum"},
+                     "note": "one thread-block cluster per image, bound by its chain of steps; bytes are the algorithmic minimum"},
         "kernels": kinfo, "clocks": ck,
         "gpu": torch.cuda.get_device_name(dev), "host_cores": os.cpu_count(), "seed": 4,
     }
