@@ -41,8 +41,9 @@
 // on one lane), groups of large balls and joined groups on a whole CTA.
 //
 // What a phase cannot hold (a group beyond its step budget or queue, more
-// roots or steps than the tables take) stops the kernel with a flag; the
-// caller then runs the one-CTA loop of invade.cu from the start.
+// roots or steps than the tables take) stops the kernel before anything of the
+// phase is stamped; the caller then lets the one-CTA loop of invade.cu go on
+// from the steps taken.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -820,7 +821,7 @@ __device__ void flood_body(const Flood &f, const int T, const int c)
     FloodCtl *ctl = f.ctl;
 
     // ---- set-up: clear the tables, then state, sequence and value counts
-    if (c == 0 && tid == 0) f.out[1] = kFloodGiveUp;   // until the end is reached
+    if (c == 0 && tid == 0) { f.out[0] = -1; f.out[1] = kFloodGiveUp; }   // until the end is reached
     for (int64_t i = gt; i <= f.maxd; i += GT) f.cnt[i] = 0;
     for (int64_t i = gt; i < f.plane_words; i += GT) f.plane[i] = 0u;
     {
@@ -1464,9 +1465,13 @@ void ibip_flood_fill(Flood *f, const int32_t *dt2, ibip_dims d, int inlet, const
     f->cancel = nullptr;
     f->rec = nullptr;
     // A group longer than this is a serial chain that the one-CTA loop runs
-    // faster: a long group takes ~2 us a step, the loop 0.3-0.4 us a step on
-    // all the steps, of which there is one for 15-25 voxels.
-    f->budget = (int)std::min<int64_t>(std::max<int64_t>(N / 64, 4096), 1 << 18);
+    // faster: a long group takes 2-4 us a step (more with thousands in its
+    // queue), the loop 0.3-0.7 us a step on all the steps.  The longest group
+    // of the 512^3 blobs has under 14,478 steps.  Packs of 290^3-350^3 and
+    // porosity 0.36-0.45, whose last bursts outgrow the queue, take 1,787,
+    // 2,484, 1,959 and 2,410 ms so (the loop alone 1,746, 2,396, 1,955 and
+    // 2,649); with 16,384 entries and N / 256 steps 397, 2,698, 2,173 and 2,402.
+    f->budget = (int)std::min<int64_t>(std::max<int64_t>(N / 1024, 4096), 1 << 18);
 }
 
 int ibip_flood_launch_grid(ibip_ctx *ctx, const Flood &f, cudaStream_t s)

@@ -1835,13 +1835,14 @@ bool l1_fits_smem(const Inv &a)
 // One image by value phases (flood.cu): on the whole GPU when the context has
 // it to itself and the image is large enough to fill it, else on one
 // thread-block cluster.  kFloodGiveUp: the run outgrew its tables and the
-// one-CTA loop has to take the image from the start (a resumed run cannot:
-// its sequence image is partly written by then, so it is copied back first).
+// one-CTA loop goes on from the *k_done steps taken (phases are stamped whole),
+// or takes the image from the start if a barrier gave up (*k_done < 0; the
+// sequence image of a resumed run is then copied back first).
 // The tables share the scratch slots of that loop, of the EDT passes and of
 // the widest path, none of which runs meanwhile.
 int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps, int32_t *seq,
               int32_t *step_r2, int32_t *step_centre, int64_t cap, int maxd, int npore, const uint8_t *mask, int resume,
-              int64_t k0, int64_t *h_out)
+              int64_t k0, int64_t *h_out, int64_t *k_done)
 {
     cudaStream_t s = ctx->stream;
     const int64_t N = nvox(d);
@@ -1898,7 +1899,9 @@ int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t
     if (e != cudaSuccess) return ibip_cuda_status(e);
     if (ho[1] == kFloodGiveUp) {
         ibip_prof_begin(ctx, IBIP_K_RANK);
-        if (resume) cudaMemcpyAsync(seq, keep, (size_t)N * sizeof(int32_t), cudaMemcpyDeviceToDevice, ctx->stream);
+        *k_done = ho[0];
+        if (resume && *k_done < 0)
+            cudaMemcpyAsync(seq, keep, (size_t)N * sizeof(int32_t), cudaMemcpyDeviceToDevice, ctx->stream);
         return kFloodGiveUp;
     }
     for (int i = 0; i < kNOut; i++) h_out[i] = 0;
@@ -2015,9 +2018,13 @@ int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, i
         return ibip_cuda_status(ibip_sync(ctx, s));
     }
     if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf)) {
+        int64_t done = -1;
         const int st = flood_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, mask, resume,
-                                 k0, h_out);
+                                 k0, h_out, &done);
         if (st != kFloodGiveUp) return st;
+        if (done >= 0)
+            return loop_run(ctx, dt2, d, inlet, max_steps - (done - k0), seq, step_r2, step_centre, cap, maxd, npore, hasinf,
+                            mask, 1, done, h_out);
     }
     return loop_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, hasinf, mask, resume, k0,
                     h_out);
@@ -2063,6 +2070,7 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
     int top = 1;   // largest finite dt2 of the images run by phases
     std::vector<FloodSizes> z(n);
     std::vector<int> idx, single;   // images run by phases, and by the one-CTA loop
+    std::vector<int64_t> taken(n, -1);   // steps of the phases of those that gave up
     int64_t pore_total = 0;
     for (int j = 0; j < n; j++) {
         maxd[j] = h[3 * j]; npore[j] = h[3 * j + 1]; hasinf[j] = h[3 * j + 2];
@@ -2142,7 +2150,11 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
                     std::atomic_thread_fence(std::memory_order_acquire);   // the record, then its flag
                     seen[q] = 1;
                     nseen++;
-                    if (hd[q].status == kFloodGiveUp) { single.push_back(idx[q]); continue; }
+                    if (hd[q].status == kFloodGiveUp) {
+                        taken[idx[q]] = hd[q].steps;
+                        single.push_back(idx[q]);
+                        continue;
+                    }
                     it[idx[q]].n_steps = hd[q].steps;
                     it[idx[q]].status = hd[q].status;
                     done.push_back(idx[q]);
@@ -2165,7 +2177,11 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
             const cudaError_t e = ibip_sync(ctx, s);
             if (e != cudaSuccess) return ibip_cuda_status(e);
             for (int q = 0; q < m; q++) {
-                if (ho[2 * q + 1] == kFloodGiveUp) { single.push_back(idx[q]); continue; }
+                if (ho[2 * q + 1] == kFloodGiveUp) {
+                    taken[idx[q]] = ho[2 * q];
+                    single.push_back(idx[q]);
+                    continue;
+                }
                 it[idx[q]].n_steps = ho[2 * q];
                 it[idx[q]].status = (int)ho[2 * q + 1];
             }
@@ -2178,8 +2194,9 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
     for (int j : single) {
         int64_t out[kNOut] = {0};
         ibip_prof_begin(ctx, IBIP_K_RANK);
-        const int st = loop_run(ctx, it[j].dt2, it[j].d, it[j].inlet, it[j].max_steps, it[j].seq, it[j].step_r2,
-                                it[j].step_centre, it[j].cap, maxd[j], npore[j], hasinf[j], nullptr, 0, 0, out);
+        const int64_t k = std::max<int64_t>(taken[j], 0);
+        const int st = loop_run(ctx, it[j].dt2, it[j].d, it[j].inlet, it[j].max_steps - k, it[j].seq, it[j].step_r2,
+                                it[j].step_centre, it[j].cap, maxd[j], npore[j], hasinf[j], nullptr, taken[j] >= 0, k, out);
         if (st) return st;
         it[j].n_steps = out[0];
         it[j].status = (int)out[1];
