@@ -761,8 +761,11 @@ int ibip_invade_batched(ibip_ctx *ctx, int32_t n, ibip_job *jobs)
     if (st) return st;
     // Trapping and curves run in two groups: the images whose invasion is
     // done while the last few still run (on a second stream, overlapping
-    // them), then the rest.  All scratch they use is sized first, so nothing
-    // is reallocated while kernels run.
+    // them), then the rest.  The scratch they use is sized first, so that
+    // nothing is reallocated while kernels run (but for an image whose basins
+    // are more than an eighth of its voxels: that waits for the second stream,
+    // and the invasions running use none of it).  Images that the phases leave
+    // to the one-CTA loop run after both streams are done.
     if (!ctx->stream2 && cudaStreamCreateWithFlags(&ctx->stream2, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         ctx->stream2 = nullptr;

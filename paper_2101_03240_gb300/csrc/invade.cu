@@ -2189,7 +2189,10 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
     } else {
         ibip_prof_end(ctx, IBIP_K_RANK);
     }
-    const cudaError_t e = ibip_sync(ctx, s);
+    cudaError_t e = ibip_sync(ctx, s);
+    // what `early` queued on the second stream reads basins and scans in slots
+    // that the loop writes (SC_OKEY, SC_SCAN)
+    if (e == cudaSuccess && !single.empty() && ctx->stream2) e = ibip_sync(ctx, ctx->stream2);
     if (e != cudaSuccess) return ibip_cuda_status(e);
     for (int j : single) {
         int64_t out[kNOut] = {0};
