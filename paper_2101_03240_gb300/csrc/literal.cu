@@ -407,7 +407,8 @@ constexpr int kWT = 512;            // threads of the walk
 constexpr int kWalkVals = 4095;     // largest squared distance it takes
 constexpr int kSoloPts = 21;        // points of a step run on one warp (four passes of 32 lanes)
 constexpr int kCtaPts = 512;        // points of a step run on one CTA
-constexpr int kWalkRing = 16;       // last entries of each list kept in shared memory (fewer for large values)
+constexpr int kWalkRing = 16;       // last entries of each list kept in shared memory (fewer for large values);
+                                    // read by steps that take no more points than that
 
 // The state and step images of the walk have a border of one solid voxel, so
 // that a neighbour is an offset and no step needs coordinates: voxel
@@ -675,7 +676,9 @@ __global__ void __launch_bounds__(kWT, 1) k_walk(Walk a)
                             const int i = lane + 32 * j, q = i / 6, dir = i - 6 * q, p = h + q;
                             v[j] = -1;
                             if (q >= n) continue;
-                            const int u = e - p <= rsz ? ring[t * rsz + (p & rm)] : __ldcg(list + start[t] + p);
+                            // (places rsz apart share a slot of the ring, and the threads that queue
+                            // them are not ordered: more than rsz points come from the list)
+                            const int u = n <= rsz ? ring[t * rsz + (p & rm)] : __ldcg(list + start[t] + p);
                             if (dir == 0) when[u] = (int32_t)k;
                             v[j] = u + offset(dir);
                         }
