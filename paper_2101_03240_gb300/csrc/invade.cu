@@ -1912,7 +1912,6 @@ int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t
     h_out[kErrSlot] = ho[4];
     h_out[kErrSlot + 1] = ho[5];
 #endif
-    if (h_out[1] == IBIP_ERR_CANCELLED && ctx->h_cancel) *ctx->h_cancel = 0;   // the request is served
     return IBIP_OK;
 }
 
@@ -1979,7 +1978,6 @@ int loop_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t 
     cudaError_t e = ibip_sync(ctx, s);
     if (e != cudaSuccess) return ibip_cuda_status(e);
     for (int i = 0; i < kNOut; i++) h_out[i] = ho[i];
-    if (h_out[1] == IBIP_ERR_CANCELLED && ctx->h_cancel) *ctx->h_cancel = 0;   // the request is served
     return IBIP_OK;
 }
 
@@ -2017,17 +2015,19 @@ int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, i
         h_out[1] = IBIP_OK;
         return ibip_cuda_status(ibip_sync(ctx, s));
     }
-    if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf)) {
-        int64_t done = -1;
-        const int st = flood_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, mask, resume,
-                                 k0, h_out, &done);
-        if (st != kFloodGiveUp) return st;
-        if (done >= 0)
-            return loop_run(ctx, dt2, d, inlet, max_steps - (done - k0), seq, step_r2, step_centre, cap, maxd, npore, hasinf,
-                            mask, 1, done, h_out);
-    }
-    return loop_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, hasinf, mask, resume, k0,
-                    h_out);
+    int64_t done = -1;
+    int st = kFloodGiveUp;
+    if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf))
+        st = flood_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, mask, resume, k0, h_out,
+                       &done);
+    if (st == kFloodGiveUp && done >= 0)
+        st = loop_run(ctx, dt2, d, inlet, max_steps - (done - k0), seq, step_r2, step_centre, cap, maxd, npore, hasinf, mask, 1,
+                      done, h_out);
+    else if (st == kFloodGiveUp)
+        st = loop_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, hasinf, mask, resume, k0,
+                      h_out);
+    if (st == IBIP_OK && h_out[1] == IBIP_ERR_CANCELLED && ctx->h_cancel) *ctx->h_cancel = 0;   // the request is served
+    return st;
 }
 
 int ibip_stats_launch(ibip_ctx *ctx, const int32_t *dt2, int64_t N, int *stats)

@@ -81,3 +81,20 @@ def test_mixed_sizes_some_on_the_loop(ibip):
     want = [alone(ctx, d, 2, 3) for d in dev]
     for got, w in zip(ctx.invade_batched(dev, 2, 3), want):
         same(got, w)
+
+
+def test_cancel_covers_every_image_on_the_loop(ibip):
+    """A request made before the call stops the images of the phases and all
+    of those left to the loop, and is served once."""
+    rng = np.random.default_rng(12)
+    imgs = [np.ones((20, 22, 18), np.uint8), S.blobs((23, 22, 18), 2.0, 0.6, rng), np.ones((9, 30, 33), np.uint8),
+            np.ones((12, 12, 40), np.uint8)]
+    dev = [cuda(a) for a in imgs]
+    ctx = ibip.Context(0)
+    ctx.cancel(True)
+    res = ctx.invade_batched(dev, 0, trapping=False, curve=False, check=False)
+    assert all(r["status"] == ibip.ERR_CANCELLED and r["K"] == 0 for r in res)
+    res = ctx.invade_batched(dev, 0, trapping=False, curve=False)
+    for a, r in zip(imgs, res):
+        assert r["status"] == ibip.OK
+        assert np.array_equal(r["seq"].cpu().numpy(), O.invade(a, O.edt(a), inlet=0)[0])
