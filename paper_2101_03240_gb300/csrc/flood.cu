@@ -1464,14 +1464,19 @@ void ibip_flood_fill(Flood *f, const int32_t *dt2, ibip_dims d, int inlet, const
     f->out = m.out;
     f->cancel = nullptr;
     f->rec = nullptr;
-    // A group longer than this is a serial chain that the one-CTA loop runs
-    // faster: a long group takes 2-4 us a step (more with thousands in its
-    // queue), the loop 0.3-0.7 us a step on all the steps.  The longest group
-    // of the 512^3 blobs has under 14,478 steps.  Packs of 290^3-350^3 and
-    // porosity 0.36-0.45, whose last bursts outgrow the queue, take 1,787,
-    // 2,484, 1,959 and 2,410 ms so (the loop alone 1,746, 2,396, 1,955 and
-    // 2,649); with 16,384 entries and N / 256 steps 397, 2,698, 2,173 and 2,402.
-    f->budget = (int)std::min<int64_t>(std::max<int64_t>(N / 1024, 4096), 1 << 18);
+    // A longer group is a serial chain that the one-CTA loop runs faster: a
+    // long group takes 2-4 us a step (more with thousands in its queue), the
+    // loop 0.4-1.1 us, but on all the steps.  Packs of 100^3-220^3 have a group
+    // of up to 0.8 % of their pore voxels and run 3-8 times faster by phases
+    // (117^3, porosity 0.43: 5,281 steps, 35 ms against 104; 160^3, 0.40: 11,681,
+    // 70 against 280; 220^3, 0.40: 28,796, 170 against 739); at 290^3 the share
+    // falls (0.36: 36,830 steps, 0.4 %, 379 ms against 1,876; 512^3 blobs: under
+    // 14,478).  What gives up pays for the steps once more: 30 ms of the loop's
+    // 1,739 at 290^3 and 0.40, 20 of 3,083 at 350^3 (both by the queue).  Small
+    // images get a larger share, noise of single voxels (a group of most steps,
+    // whatever the size) bounds it: 32^3 takes 19 ms so and 27 ms with 4,096
+    // steps, the loop alone 18.
+    f->budget = std::min(std::max(npore / 96, std::min(npore / 32, 4096)), 40960);
 }
 
 int ibip_flood_launch_grid(ibip_ctx *ctx, const Flood &f, cudaStream_t s)
