@@ -347,7 +347,9 @@ typedef struct {
  * saturation / Pc curve (Sections 2.2.1-2.2.2; computed from seq_out when
  * trapping ran, else from seq) when `sat_per_step` is given.  The
  * invasions of all images run in one launch, one thread-block cluster per
- * image, largest first; results equal the per-image calls bit for bit.
+ * image, largest first (images without solid, with values above 32767 or
+ * that outgrow the phases' tables in a second one, a CTA each); results equal
+ * the per-image calls bit for bit.
  *   h_jobs: host array of n jobs (1 <= n <= 4096); n_steps and status are
  *           written back.  An image's pore count must stay below 2^25,
  *           the whole batch's below 2^31.

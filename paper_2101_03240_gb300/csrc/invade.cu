@@ -1656,6 +1656,20 @@ __global__ void __launch_bounds__(kNT, 1) k_invade(Inv a, FastDiv fd_nyz, FastDi
     invade_body<L1SMEM, PROF>(a, fd_nyz, fd_nz, gC, gD);
 }
 
+// One image per CTA (level 1 of the rank bitmap in shared memory): the images
+// of a batch that the value phases leave to the loop, side by side.
+struct InvJob {
+    Inv a;
+    FastDiv fd_nyz, fd_nz;
+    int *gC, *gD;
+};
+
+__global__ void __launch_bounds__(kNT, 1) k_invade_batch(const InvJob *__restrict__ jobs)
+{
+    const InvJob j = jobs[blockIdx.x];
+    invade_body<true, false>(j.a, j.fd_nyz, j.fd_nz, j.gC, j.gD);
+}
+
 }  // namespace
 
 // --------------------------------------------------------------- launcher --
@@ -1707,6 +1721,19 @@ JobSizes job_sizes(ibip_dims d, int npore)
     z.gl = up256((size_t)2 * npore * sizeof(int) + 64);
     z.out = up256(kNOut * sizeof(int64_t));
     return z;
+}
+
+JobMem carve(char *p, const JobSizes &z)
+{
+    JobMem m;
+    m.rank = (int32_t *)p; p += z.rank;
+    m.okey = (int2 *)p; p += z.okey;
+    m.avail = (uint32_t *)p; p += z.plane;
+    m.added = (uint32_t *)p; p += z.plane;
+    m.fb = (u64 *)p; p += z.fb;
+    m.gl = (int *)p; p += z.gl;
+    m.out = (int64_t *)p;
+    return m;
 }
 
 // The invasion kernel's view of one image, its scratch carved as in `mem`.
@@ -2039,6 +2066,62 @@ int ibip_stats_launch(ibip_ctx *ctx, const int32_t *dt2, int64_t N, int *stats)
 
 // ------------------------------------------------------------- batched --
 
+// The images `single` of a batch on the one-CTA loop, in one launch, largest
+// first: rank sorts one after the other, then a CTA each (four 64^3 images of
+// a chain each: 159 ms, one after the other 533).  taken: steps the phases
+// took of an image, negative if none.  Nothing else runs meanwhile, so the
+// tables take the place of the phases'.
+static int loop_batch(ibip_ctx *ctx, IbipBatchItem *it, std::vector<int> &single, const std::vector<int64_t> &taken,
+                      const std::vector<int> &maxd, const std::vector<int> &npore, const std::vector<int> &hasinf)
+{
+    cudaStream_t s = ctx->stream;
+    const int m = (int)single.size();
+    std::stable_sort(single.begin(), single.end(), [&](int a, int b) { return npore[a] > npore[b]; });
+    size_t total = 0;
+    for (int j : single) total += job_sizes(it[j].d, npore[j]).total();
+    char *arena = (char *)ibip_scratch(ctx, SC_BARENA, total + 256);
+    InvJob *djobs = (InvJob *)ibip_scratch(ctx, SC_BJOBS, (size_t)m * sizeof(InvJob));
+    if (!arena || !djobs) return IBIP_ERR_OOM;
+    ibip_prof_begin(ctx, IBIP_K_RANK);
+    std::vector<InvJob> jobs(m);
+    size_t off = 0, dyn = 0;
+    for (int q = 0; q < m; q++) {
+        const int j = single[q];
+        const JobSizes z = job_sizes(it[j].d, npore[j]);
+        const JobMem mem = carve(arena + off, z);
+        off += z.total();
+        const int64_t k = std::max<int64_t>(taken[j], 0);
+        InvJob &J = jobs[q];
+        const int st = invade_setup(ctx, it[j].dt2, it[j].d, it[j].inlet, it[j].max_steps - k, it[j].seq, it[j].step_r2,
+                                    it[j].step_centre, it[j].cap, maxd[j], npore[j], hasinf[j], mem, &J.a, nullptr,
+                                    taken[j] >= 0, k);
+        if (st) return st;
+        J.a.cancel = ctx->d_cancel;
+        J.fd_nyz = make_fastdiv((uint32_t)it[j].d.ny * (uint32_t)it[j].d.nz);
+        J.fd_nz = make_fastdiv((uint32_t)it[j].d.nz);
+        J.gC = mem.gl;
+        J.gD = mem.gl + npore[j];
+        dyn = std::max(dyn, invade_dyn_smem(J.a, true));
+    }
+    cudaMemcpyAsync(djobs, jobs.data(), (size_t)m * sizeof(InvJob), cudaMemcpyHostToDevice, s);
+    ibip_prof_end(ctx, IBIP_K_RANK);
+    ibip_prof_begin(ctx, IBIP_K_INVADE);
+    allow_max_dyn_smem((const void *)k_invade_batch);
+    k_invade_batch<<<m, kNT, dyn, s>>>(djobs);
+    IBIP_LAUNCH(ctx);
+    ibip_prof_end(ctx, IBIP_K_INVADE);
+    int64_t *ho = (int64_t *)ctx->h_pinned;
+    for (int q = 0; q < m; q++)
+        cudaMemcpyAsync(ho + 2 * q, jobs[q].a.out, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    const cudaError_t e = ibip_sync(ctx, s);
+    if (e != cudaSuccess) return ibip_cuda_status(e);
+    for (int q = 0; q < m; q++) {
+        it[single[q]].n_steps = ho[2 * q];
+        it[single[q]].status = (int)ho[2 * q + 1];
+    }
+    return IBIP_OK;
+}
+
 int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarly early, void *user)
 {
     cudaStream_t s = ctx->stream;
@@ -2194,15 +2277,9 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
     // that the loop writes (SC_OKEY, SC_SCAN)
     if (e == cudaSuccess && !single.empty() && ctx->stream2) e = ibip_sync(ctx, ctx->stream2);
     if (e != cudaSuccess) return ibip_cuda_status(e);
-    for (int j : single) {
-        int64_t out[kNOut] = {0};
-        ibip_prof_begin(ctx, IBIP_K_RANK);
-        const int64_t k = std::max<int64_t>(taken[j], 0);
-        const int st = loop_run(ctx, it[j].dt2, it[j].d, it[j].inlet, it[j].max_steps - k, it[j].seq, it[j].step_r2,
-                                it[j].step_centre, it[j].cap, maxd[j], npore[j], hasinf[j], nullptr, taken[j] >= 0, k, out);
+    if (!single.empty()) {
+        const int st = loop_batch(ctx, it, single, taken, maxd, npore, hasinf);
         if (st) return st;
-        it[j].n_steps = out[0];
-        it[j].status = (int)out[1];
     }
     return first_err;
 }

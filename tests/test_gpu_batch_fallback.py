@@ -2,6 +2,8 @@
 value phases give up, images without solid) while the trapping and the curves
 of the others are under way on the second stream: every output of every image
 equals the calls made for it alone (Sections 2.1-2.2)."""
+import time
+
 import numpy as np
 import pytest
 
@@ -98,3 +100,19 @@ def test_cancel_covers_every_image_on_the_loop(ibip):
     for a, r in zip(imgs, res):
         assert r["status"] == ibip.OK
         assert np.array_equal(r["seq"].cpu().numpy(), O.invade(a, O.edt(a), inlet=0)[0])
+
+
+def test_images_on_the_loop_run_side_by_side(ibip):
+    """Sixteen chains in a batch take far less than sixteen times one."""
+    ctx = ibip.Context(0)
+    dev = [cuda(chain(60 + i)) for i in range(16)]
+
+    def seconds(imgs):
+        ctx.invade_batched(imgs, 0, trapping=False, curve=False)
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        ctx.invade_batched(imgs, 0, trapping=False, curve=False)
+        torch.cuda.synchronize()
+        return time.perf_counter() - t
+
+    assert seconds(dev) < 0.5 * 16 * seconds(dev[:1])
