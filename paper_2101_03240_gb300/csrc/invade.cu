@@ -8,7 +8,8 @@
 // An invasion runs by value phases (flood.cu) on the whole GPU or on one
 // thread-block cluster, a batch on one cluster per image; set-up, launch and
 // completion are here.  Traced runs, images without solid, values above
-// 32767 and runs the phases give up take the loop below.
+// 32767, runs the phases give up and runs that are faster so (loop_is_faster)
+// take the loop below.
 //
 // The one-CTA loop:
 //  * Rank: pore voxels are ranked once by (dt2 descending, index ascending),
@@ -37,6 +38,7 @@
 #include <thread>
 #include <vector>
 #include <climits>
+#include <cmath>
 
 #include "common.cuh"
 #include "flood.cuh"
@@ -2008,6 +2010,23 @@ int loop_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t 
     return IBIP_OK;
 }
 
+// Whether the loop beats the phases on one image.
+//  * Few large balls: a phase costs its barriers (~25 us on a cluster) however
+//    few steps it has, and one large ball after the other leaves nothing to run
+//    in parallel.  The measure is the pore volume in largest balls (but for a
+//    factor of 4): below 24 the loop is faster, above ~35 the phases are.
+//    phases / loop at 64^3 with 10 and 100 solid voxels (2.6, 21) 3.28 / 1.24 and
+//    3.04 / 1.98 ms, 128^3 with 100 (24) 11.96 / 7.97, 12^3-16^3 samples (7-16)
+//    0.50-0.65 / 0.34-0.57; 200^3 with 100 (29) 25.1 / 25.6, 64^3 pack of radius 8
+//    (45) 2.73 / 6.22, 48^3 blobs (92) 1.87 / 2.35.
+//  * Short continuations: the phases take the whole phase that a step limit
+//    falls in.  1,000 steps more of the 200^3 pack 2.5-3.7 / 0.8-0.9 ms, 10,000
+//    1.9-3.0 / 2.9-3.1; of the 512^3 blobs 5.6-7.6 / 5.2-7.1.
+bool loop_is_faster(int64_t npore, int maxd, int resume, int64_t max_steps)
+{
+    return (double)npore < 24.0 * maxd * std::sqrt((double)maxd) || (resume && max_steps <= 4096);
+}
+
 }  // namespace
 
 int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t max_steps,
@@ -2044,7 +2063,7 @@ int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, i
     }
     int64_t done = -1;
     int st = kFloodGiveUp;
-    if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf))
+    if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf) && !loop_is_faster(npore, maxd, resume, max_steps))
         st = flood_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, mask, resume, k0, h_out,
                        &done);
     if (st == kFloodGiveUp && done >= 0)
