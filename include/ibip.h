@@ -614,9 +614,9 @@ IBIP_API int ibip_edt_tiles(ibip_ctx *ctx, ibip_dims dims, int *h_z_warps, int *
  * it starts; on = 0 withdraws the request.  Safe to call from another host
  * thread while ibip_invade / ibip_invade_ex / ibip_invade_batched block.
  * The flag lives in host-mapped memory; the invasion kernel reads it every
- * 4 value phases (the one-CTA loop every 16 batches of its main loop and
- * every 64 of its single-voxel loop) and stops before the next phase or
- * batch: the call returns
+ * 4 value phases and every 512 steps of a phase's long group (the one-CTA
+ * loop every 16 batches of its main loop and every 64 of its single-voxel
+ * loop) and stops before anything more is stamped: the call returns
  * IBIP_ERR_CANCELLED with *h_n_steps = k, and seq, step_r2 and step_centre
  * hold a valid invasion of k steps, which ibip_invade_ex(resume = 1)
  * continues to the same result as an uninterrupted call.  Serving the

@@ -10,7 +10,7 @@ constexpr int kFloodGiveUp = -100;     // status of a run that outgrew its table
 // Counters of one image, zero before the launch.
 struct FloodCtl {
     unsigned int bar;   // arrivals at the grid barrier
-    int fail;           // a group or a barrier gave up
+    int fail;           // a group (1) or a barrier (2) gave up, or a group was cancelled (3)
     int R;              // roots of the phase
     int nlog;           // log slots taken
     int next, nextC;    // work counters of the round (warps, CTAs)
