@@ -56,10 +56,33 @@ constexpr int kNOut = kInvStats;   // int64 outputs of the invasion kernel
 // 5.1 / 5.6 ms; the line is the middle).
 constexpr int64_t kFloodGridVox = 1 << 19;
 constexpr int kFloodCluster = 16;   // CTAs of one image on a cluster
-// CTAs of each image of a batch of n: fewer when the images fill the GPU
-// (96 images of 32^3-160^3, invasion only: clusters of 1, 2, 4, 8, 16 take
-// 185, 103, 68, 54, 86 ms).
-int flood_batch_cluster(int n) { return n <= 24 ? 16 : n <= 128 ? 8 : 4; }
+// CTAs of each image of a batch (vox: the images' voxels): many for a few
+// large images, whose longest run is what the batch waits for; few for many
+// small ones, which then wait in fewer waves (a cluster of 8 leaves room for 19
+// images, one of 1 for 152).  An image of N voxels takes about 5e-5 N / c +
+// 1.5e-3 N^0.56 + 0.06 ms on c CTAs: its voxels, which the CTAs share, and its
+// chain of steps, which they do not.  The batch is put at the square root of
+// the squares' sum of its longest image and of all images over the room for
+// them.  Of 39 batches measured with every size (1-400 images of 16^3-160^3,
+// alike and mixed) 32 get the best size and the others one at most 20 % slower;
+// 128 of 48^3 take 10.4 / 10.2 / 13.4 / 22.8 / 42.1 ms on 1 / 2 / 4 / 8 / 16, 64 of 100^3
+// 69 / 43 / 35 / 49 / 73, 96 of 32^3-160^3 279 / 174 / 120 / 90 / 85.
+int flood_batch_cluster(const std::vector<int64_t> &vox, int sm_count)
+{
+    int best = 1;
+    double least = 0.0;
+    for (int c = 1; c <= kFloodCluster; c *= 2) {
+        double longest = 0.0, sum = 0.0;
+        for (int64_t n : vox) {
+            const double t = 5e-5 * (double)n / c + 1.5e-3 * std::pow((double)n, 0.56) + 0.06;
+            longest = std::max(longest, t);
+            sum += t;
+        }
+        const double room = 1.15 * sum / std::max(sm_count / c, 1), all = longest * longest + room * room;
+        if (c == 1 || all < least) { least = all; best = c; }
+    }
+    return best;
+}
 static_assert(64 + kNOut * sizeof(long long) <= kSmallBytes, "output slot too small");
 
 typedef unsigned long long u64;
@@ -2234,7 +2257,9 @@ int ibip_invade_batch_run(ibip_ctx *ctx, int n, IbipBatchItem *it, IbipBatchEarl
             for (int q = 0; q < m; q++) hd[q].done = 0;
         ibip_prof_end(ctx, IBIP_K_RANK);
         ibip_prof_begin(ctx, IBIP_K_INVADE);
-        const int st = ibip_flood_launch_clusters(ctx, djobs, m, top, flood_batch_cluster(m), s);
+        std::vector<int64_t> vox(m);
+        for (int q = 0; q < m; q++) vox[q] = nvox(it[idx[q]].d);
+        const int st = ibip_flood_launch_clusters(ctx, djobs, m, top, flood_batch_cluster(vox, ctx->sm_count), s);
         if (st) return st;
         ibip_prof_end(ctx, IBIP_K_INVADE);
         if (hd) {
