@@ -1482,10 +1482,11 @@ void ibip_flood_fill(Flood *f, const int32_t *dt2, ibip_dims d, int inlet, const
     // falls (0.36: 36,830 steps, 0.4 %, 379 ms against 1,876; 512^3 blobs: under
     // 14,478).  What gives up pays for the steps once more: 30 ms of the loop's
     // 1,739 at 290^3 and 0.40, 20 of 3,083 at 350^3 (both by the queue).  Small
-    // images get a larger share, noise of single voxels (a group of most steps,
-    // whatever the size) bounds it: 32^3 takes 19 ms so and 27 ms with 4,096
+    // images get a larger share (16^3-32^3 packs of narrow pores have groups of
+    // 250-500 steps and more), noise of single voxels (a group of most steps,
+    // whatever the size) bounds it: 32^3 takes 21 ms so and 27 ms with 4,096
     // steps, the loop alone 18.
-    f->budget = std::min(std::max(npore / 96, std::min(npore / 32, 4096)), 40960);
+    f->budget = std::min(std::max(npore / 96, std::min(std::max(npore / 32, 1024), 4096)), 40960);
 }
 
 int ibip_flood_launch_grid(ibip_ctx *ctx, const Flood &f, cudaStream_t s)

@@ -36,3 +36,17 @@ def test_taken_whole(ibip, edge, porosity, seed):
         assert np.array_equal(r2.cpu().numpy(), rr2) and np.array_equal(cen.cpu().numpy(), rcen)
     out = ctx.invade_batched([dev, dev[:40].contiguous()], 0, trapping=False, curve=False)[0]
     assert out["K"] == K and np.array_equal(out["seq"].cpu().numpy(), rseq)
+
+
+def test_small_packs_taken_whole(ibip):
+    """Groups of a few hundred steps in 24^3 and 32^3 packs."""
+    ctx = ibip.Context(0)
+    for n, m in ((24, 40), (32, 16)):
+        for seed in range(m):
+            img = S.sphere_pack((n,) * 3, 4, 0.42, np.random.default_rng(seed))
+            d = O.edt(img)
+            if img.sum() < 30 * float(d.max()) ** 1.5:
+                continue   # few large balls: the loop's by rule
+            seq = ctx.invade(torch.from_numpy(img).cuda(), torch.from_numpy(d).cuda())[0]
+            assert ctx.invade_stats()["items"] == 0
+            assert np.array_equal(seq.cpu().numpy(), O.invade(img, d, inlet=0)[0])
