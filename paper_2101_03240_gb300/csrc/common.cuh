@@ -66,9 +66,12 @@ struct ibip_ctx {
     // Kernels share the device with other streams: no cooperative launches
     // (the invasion runs on one cluster).
     int no_coop;
+    // CTAs of an invasion of fewer than 2^20 voxels that runs on a cluster
+    // (0: 16).
+    int small_cluster;
     // Server slots: the invasion kernel goes to this stream (of the
     // device's highest priority, owned by the context, with an event that
-    // orders it after the work queued before it), so that its one CTA is
+    // orders it after the work queued before it), so that its cluster is
     // placed ahead of the waiting blocks of other jobs' wide kernels; null
     // elsewhere.
     cudaStream_t stream_inv;

@@ -1942,7 +1942,8 @@ int flood_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t
         s = ctx->stream_inv;
     }
     const int st = grid ? ibip_flood_launch_grid(ctx, f, s)
-                        : ibip_flood_launch_clusters(ctx, (const Flood *)(c + kCtl), 1, maxd, kFloodCluster, s);
+                        : ibip_flood_launch_clusters(ctx, (const Flood *)(c + kCtl), 1, maxd,
+                                                     ctx->small_cluster && N < (1 << 20) ? ctx->small_cluster : kFloodCluster, s);
     if (st) return st;
     ibip_prof_end(ctx, IBIP_K_INVADE);
     int64_t *ho = (int64_t *)ctx->h_pinned;

@@ -237,9 +237,9 @@ int ibip_server_create(ibip_server **out, ibip_ctx *ctx, size_t mem_budget, int 
         st = IBIP_ERR_OOM;
     }
     S->alloc = RangeAlloc(S->arena ? mem_budget : 0);
-    // every slot's wide kernels (EDT, rank sort, widest path, curve) queue
-    // at the device's lowest stream priority and its one-CTA invasion at the
-    // highest: when an SM frees up, a waiting invasion is placed before more
+    // every slot's wide kernels (EDT, curve) queue at the device's lowest
+    // stream priority, its invasion (one cluster) and widest path at the
+    // highest: when SMs free up, a waiting invasion is placed before more
     // blocks of the other jobs' wide kernels
     int prio_low = 0, prio_high = 0;
     if (cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high) != cudaSuccess) {
@@ -268,6 +268,11 @@ int ibip_server_create(ibip_server **out, ibip_ctx *ctx, size_t mem_budget, int 
         st = ibip_create(&c, S->device, s);
         if (st) { cudaStreamDestroy(s); cudaStreamDestroy(si); cudaEventDestroy(ev); cudaEventDestroy(evb); break; }
         c->no_coop = 1;
+        // nine clusters of 16 fit the GPU at once: with more slots than 16 small
+        // jobs take smaller ones (60 requests of 48^3, 24 / 64 slots: 21.9 / 22.5 ->
+        // 13.8 / 12.2 ms; of 64^3 21.8 / 23.5 -> 15.0 / 13.0), large ones, whose own
+        // time counts, do not (mixed 64^3-200^3: 67 ms, 74 and 104 with 8 and 4)
+        c->small_cluster = max_slots <= 16 ? 16 : max_slots <= 32 ? 8 : 4;
         c->stream_inv = si;   // owned by the context from here on
         c->ev_inv = ev;
         c->ev_block = evb;
