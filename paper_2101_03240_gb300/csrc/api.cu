@@ -789,7 +789,7 @@ int ibip_invade_batched(ibip_ctx *ctx, int32_t n, ibip_job *jobs)
     P.M = mm_total ? (int32_t *)ibip_scratch(ctx, SC_MM, (size_t)mm_total * sizeof(int32_t)) : nullptr;
     // the widest path's tables: basins are a few percent of the voxels
     const size_t basins = (size_t)mm_total / 8 + 1024;
-    if ((mm_total && (!P.M || !ibip_scratch(ctx, SC_TILE, ibip_maximin_table_bytes(ctx, n, mm_total)) ||
+    if ((mm_total && (!P.M || !ibip_scratch(ctx, SC_TILE, ibip_maximin_table_bytes(n, mm_total)) ||
                       !ibip_scratch(ctx, SC_OKEY, basins * 8) || !ibip_scratch(ctx, SC_HIST, basins * 8) ||
                       !ibip_scratch(ctx, SC_RANK, (size_t)mm_total * 4) ||
                       !ibip_scratch(ctx, SC_G2, (size_t)mm_total * 4) ||
@@ -866,7 +866,7 @@ const char *ibip_status_string(int s)
     case IBIP_ERR_CUDA: return "CUDA runtime error";
     case IBIP_ERR_OOM: return "out of device memory";
     case IBIP_ERR_STEP_LIMIT: return "step limit reached with candidates left";
-    case IBIP_ERR_NOT_CONVERGED: return "propagation did not converge within its round or activation limit";
+    case IBIP_ERR_NOT_CONVERGED: return "a device loop did not end within its round or step limit";
     case IBIP_ERR_CANCELLED: return "cancelled";
     case IBIP_ERR_BOUNDS: return "device index check failed";
     case IBIP_ERR_TOO_LARGE: return "image exceeds the fixed scratch of ibip_edt_noalloc (2^21 voxels)";

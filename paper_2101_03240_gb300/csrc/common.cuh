@@ -178,7 +178,7 @@ int ibip_max_launch(ibip_ctx *ctx, const int32_t *a, int64_t n, int *h_max);
 // Maximin propagation from a face through voxels with val != 0 (val == -1
 // counts as +inf).  Writes M (-1 where unreachable).
 int ibip_maximin_launch(ibip_ctx *ctx, const int32_t *val, ibip_dims d, int face, int32_t *M);
-size_t ibip_maximin_table_bytes(const ibip_ctx *ctx, int n, int64_t vox);
+size_t ibip_maximin_table_bytes(int n, int64_t vox);
 // The same for several images at once.
 struct IbipMaximinJob {
     const int32_t *val;

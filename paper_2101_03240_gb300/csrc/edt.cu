@@ -556,7 +556,8 @@ template <class Feat, class Epi, int ZW = kZWarps, int SW = kStripWarps>
 int edt_passes(ibip_ctx *ctx, Feat feat, ibip_dims d, int cap, int cap2, Epi epi, int cls)
 {
     int64_t N = nvox(d);
-    uint16_t *d1 = (uint16_t *)ibip_scratch(ctx, SC_D1, N * sizeof(uint16_t));
+    // (as many bytes as the invasion asks of the slot next: an arena gives no piece back)
+    uint16_t *d1 = (uint16_t *)ibip_scratch(ctx, SC_D1, (N + 8) * sizeof(uint16_t));
     int32_t *g2 = (int32_t *)ibip_scratch(ctx, SC_G2, N * sizeof(int32_t));
     if (!d1 || !g2) return IBIP_ERR_OOM;
     cudaStream_t s = ctx->stream;

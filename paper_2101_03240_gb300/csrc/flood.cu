@@ -105,8 +105,8 @@ __device__ __forceinline__ u64 warp_min(u64 k)
 // array's extent is recorded (the place in the code and the index), the
 // access is skipped and the call returns IBIP_ERR_BOUNDS; nothing traps.
 enum Place {
-    P_CLAIM = 1, P_STATE, P_LISTS, P_ROOT, P_LOG, P_VALUE, P_QUEUE, P_ISQ, P_HIT, P_STEP, P_PLANE, P_TODO,
-    P_VOXEL, P_CUR
+    P_CLAIM = 1, P_STATE, P_LISTS, P_ROOT, P_LOG, P_VALUE, P_QUEUE, P_ISQ, P_HIT, P_STEP, P_PLANE,
+    P_VOXEL
 };
 __device__ __forceinline__ bool in_range(FloodCtl *ctl, int64_t i, int64_t n, int place)
 {

@@ -213,6 +213,7 @@ constexpr int kChunk = 64;   // list entries a warp takes at a time
 // List entries that shrink together, at most: fewer where the list does not
 // fill the chip with that many to a warp.
 constexpr int kBlockEdges = 512;
+constexpr int kMaxSms = 256;   // SMs the tables are sized for
 
 // Every voxel pair (the voxel and its +z, +y, +x neighbour) and every face
 // voxel as an edge.  LIST: those between different roots are appended to the
@@ -469,10 +470,10 @@ __global__ void __launch_bounds__(kThreads) k_mm_value(MMWork w)
 // Table bytes for n images of vox voxels: the images, the counters and the
 // counts of the list's blocks (at most one per kBlockEdges entries, or two
 // per warp of a list that does not fill the chip).
-size_t ibip_maximin_table_bytes(const ibip_ctx *ctx, int n, int64_t vox)
+size_t ibip_maximin_table_bytes(int n, int64_t vox)
 {
     return (((size_t)n * sizeof(MMJob) + 255) & ~(size_t)255) +
-           (2 + kMaxRoundsDev + (size_t)(vox / kBlockEdges) + 1 + 64 * (size_t)ctx->sm_count) * sizeof(int);
+           (2 + kMaxRoundsDev + (size_t)(vox / kBlockEdges) + 1 + 64 * (size_t)kMaxSms) * sizeof(int);
 }
 
 // The jobs' voxels together stay below 2^31.
@@ -497,7 +498,7 @@ static int mm_group(ibip_ctx *ctx, int n, const IbipMaximinJob *jobs)
     cudaStream_t s = ctx->stream;
     const size_t jb = ((size_t)n * sizeof(MMJob) + 255) & ~(size_t)255;
     const size_t cb = (2 + kMaxRoundsDev) * sizeof(int);
-    char *t = (char *)ibip_scratch(ctx, SC_TILE, ibip_maximin_table_bytes(ctx, n, vox));
+    char *t = (char *)ibip_scratch(ctx, SC_TILE, ibip_maximin_table_bytes(n, vox));
     if (!t) return IBIP_ERR_OOM;
     MMWork w = {};
     w.jobs = (const MMJob *)t;
@@ -554,7 +555,7 @@ static int mm_group(ibip_ctx *ctx, int n, const IbipMaximinJob *jobs)
         const bool list = h[1] <= w.cap;
         bool more = h[1] > 0 && h[2] > 0;   // the list counts its unused entries too
         if (list) w.listed = h[1];
-        const int warps = ctx->sm_count * 32;
+        const int warps = std::min(ctx->sm_count, kMaxSms) * 32;
         w.block = std::min(std::max((h[1] / warps + 31) & ~31, 32), kBlockEdges);
         const int ge = (int)std::min<int64_t>(((int64_t)h[1] + kThreads - 1) / kThreads + 1, (int64_t)ctx->sm_count * 16);
         rounds = 1;

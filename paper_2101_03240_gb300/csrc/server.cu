@@ -124,7 +124,7 @@ extern "C" int64_t ibip_job_footprint(ibip_dims d, int with_dt2)
     int64_t b = 0;
     auto add = [&](int64_t x) { b += up256(x > 16 ? x : 16); };
     if (with_dt2) add(4 * N);   // dt2
-    add(2 * N);                 // EDT pass-z distances
+    add(2 * N + 16);            // EDT pass-z distances, or the phases' state
     add(4 * N);                 // EDT pass-y partial sums
     add((int64_t)kSmallBytes);
     // invasion set-up, with the pore count bounded by N
@@ -145,10 +145,10 @@ extern "C" int64_t ibip_job_footprint(ibip_dims d, int with_dt2)
     if (N + 2 > nscan) nscan = N + 2;
     for (int q = 0; q < 3; q++) add(scan_work_bytes(nscan));     // scan work, regrown at most thrice
     add(1 << 21);   // constant parts of the phase tables, which otherwise fit the entries above
-    // trapping: widest-path field, tile lists and round counters
+    // trapping: widest-path field and its tables (nodes and edges take the
+    // invasion's entries, the best edges of the basins the curve's)
     add(4 * N);
-    const int64_t nt = (int64_t)((d.nx + 3) / 4) * ((d.ny + 7) / 8) * ((d.nz + 31) / 32);
-    add(256 + (3 * nt + 2 * ((1 << 16) + 2) + 4) * 4);
+    add((int64_t)ibip_maximin_table_bytes(1, N));
     // curve: per-step histogram (steps <= pore voxels <= N)
     add(4 * (N + 2));
     return b;
