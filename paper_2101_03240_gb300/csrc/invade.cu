@@ -2043,12 +2043,16 @@ int loop_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t 
 //    3.04 / 1.98 ms, 128^3 with 100 (24) 11.96 / 7.97, 12^3-16^3 samples (7-16)
 //    0.50-0.65 / 0.34-0.57; 200^3 with 100 (29) 25.1 / 25.6, 64^3 pack of radius 8
 //    (45) 2.73 / 6.22, 48^3 blobs (92) 1.87 / 2.35.
+//  * Small images: eight samples of 24^3 (5,000-9,000 pore voxels) take 0.96 ms
+//    by phases and 0.78 on the loop on average (0.65-1.64 on the loop), eight of
+//    32^3 (12,000-22,000) 1.30 and 1.33.  (A batch keeps both kinds on the phases,
+//    where a cluster's idle time is another's.)
 //  * Short continuations: the phases take the whole phase that a step limit
 //    falls in.  1,000 steps more of the 200^3 pack 2.5-3.7 / 0.8-0.9 ms, 10,000
 //    1.9-3.0 / 2.9-3.1; of the 512^3 blobs 5.6-7.6 / 5.2-7.1.
 bool loop_is_faster(int64_t npore, int maxd, int resume, int64_t max_steps)
 {
-    return (double)npore < 24.0 * maxd * std::sqrt((double)maxd) || (resume && max_steps <= 4096);
+    return npore < 10000 || (double)npore < 24.0 * maxd * std::sqrt((double)maxd) || (resume && max_steps <= 4096);
 }
 
 }  // namespace

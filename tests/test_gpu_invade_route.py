@@ -46,12 +46,14 @@ def same(got, ref):
     (open_image((60, 70, 65), 40, 4), True),
     (open_image((100, 101, 99), 40, 5), True),
     (S.blobs((14, 12, 13), 3.0, 0.6, np.random.default_rng(1)), True),
+    (S.blobs((24, 25, 23), 1.5, 0.6, np.random.default_rng(2)), True),    # small pores, but few of them
+    (S.blobs((32, 33, 31), 1.5, 0.6, np.random.default_rng(2)), False),
     (open_image((64, 64, 64), 1000, 6), False),
     (open_image((200, 190, 201), 1000, 7), False),   # r2 >= 1024 on the phases
 ])
 def test_route_and_result(ibip, img, loop, shared):
     d = O.edt(img)
-    assert (balls(img, d) < 24.0) == loop
+    assert (balls(img, d) < 24.0 or img.sum() < 10000) == loop
     ref = O.invade(img, d, inlet=1)
     ctx = ibip.Context(0)
     ctx.set_shared_device(shared)

@@ -39,14 +39,13 @@ def test_taken_whole(ibip, edge, porosity, seed):
 
 
 def test_small_packs_taken_whole(ibip):
-    """Groups of a few hundred steps in 24^3 and 32^3 packs."""
+    """Groups of a few hundred steps in 32^3 packs."""
     ctx = ibip.Context(0)
-    for n, m in ((24, 40), (32, 16)):
-        for seed in range(m):
-            img = S.sphere_pack((n,) * 3, 4, 0.42, np.random.default_rng(seed))
-            d = O.edt(img)
-            if img.sum() < 30 * float(d.max()) ** 1.5:
-                continue   # few large balls: the loop's by rule
-            seq = ctx.invade(torch.from_numpy(img).cuda(), torch.from_numpy(d).cuda())[0]
-            assert ctx.invade_stats()["items"] == 0
-            assert np.array_equal(seq.cpu().numpy(), O.invade(img, d, inlet=0)[0])
+    for seed in range(16):
+        img = S.sphere_pack((32,) * 3, 4, 0.42, np.random.default_rng(seed))
+        d = O.edt(img)
+        if img.sum() < max(10000, 30 * float(d.max()) ** 1.5):
+            continue   # few pores or few large balls: the loop's by rule
+        seq = ctx.invade(torch.from_numpy(img).cuda(), torch.from_numpy(d).cuda())[0]
+        assert ctx.invade_stats()["items"] == 0
+        assert np.array_equal(seq.cpu().numpy(), O.invade(img, d, inlet=0)[0])
