@@ -7,7 +7,10 @@
 //   distance R that no earlier step invaded; the insertion points join the
 //   inlets and their value drops to zero.
 //
-// GPU design.  Each pore voxel is queued once, when it first becomes a
+// GPU design.  One image with solid and values up to 4095: the flood of
+// insertion points is walked first, then all spheres are stamped at once
+// (k_walk, k_walk_stamp below).  Else, and in the batched call, the schedule
+// described here.  Each pore voxel is queued once, when it first becomes a
 // candidate, into the list of its distance value ("bucket"; buckets are
 // numbered by decreasing value and own consecutive ranges of one list array
 // sized by a histogram).  A step takes the highest non-empty bucket, and
@@ -15,10 +18,11 @@
 // consumes the bucket's whole pending range, stamps the spheres of all its
 // points in parallel, then queues their uninvaded face neighbours (entries
 // queued now are examined from the next step on, as in the definition).
-// One persistent CTA of 1024 threads runs the steps, with the buckets'
-// counters and a bitmap of non-empty buckets in shared memory (up to ~10k
-// distinct values); spheres are written with fire-and-forget atomic minima,
-// so a step never waits on a read of the sequence image.
+// One thread-block cluster per image (up to 16 CTAs of 1024 threads, else one
+// CTA) runs the steps, with the buckets' counters and a bitmap of non-empty
+// buckets in shared memory (up to ~10k distinct values); spheres are written
+// with fire-and-forget atomic minima, so a step never waits on a read of the
+// sequence image.
 #include <cooperative_groups.h>
 
 #include <algorithm>
