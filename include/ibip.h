@@ -544,10 +544,9 @@ IBIP_API int ibip_profile_read(ibip_ctx *ctx, int cls, double *h_ms, int64_t *h_
  * set (ibip_invade_trace), which run a separate, timed build of the loop;
  * otherwise they read 0 (the clock reads would cost the loop about a tenth
  * of its time).  A call that ran by value phases (untraced calls, but for
- * images without solid, with values above 32767, of few pore voxels or few
- * large balls, and continuations of at most 4,096 steps) reports entries 0-2
- * and 30-34; the others describe the one-CTA loop.  Writes up to n (at most
- * 48) of:
+ * images without solid, with values above 32767 or of few steps on large
+ * balls, and continuations of at most 4,096 steps) reports entries 0-2 and
+ * 30-34; the others describe the one-CTA loop.  Writes up to n (at most 48) of:
  *   0 steps, 1 status, 2 iterations of the main loop (by phases: rounds of
  *   groups),
  *   3-5 cycles selecting, bounding (candidate shell) and committing,

@@ -92,13 +92,15 @@ __device__ __forceinline__ u64 ldcg64(const u64 *p) { return __ldcg(p); }
 
 // ------------------------------------------------------------ rank sort --
 
+template <bool ONES>   // stats[3]: voxels of value 1
 __global__ void k_stats(const int32_t *__restrict__ dt2, int64_t N, int *stats)
 {
-    int mx = 0, np = 0, inf = 0;
+    int mx = 0, np = 0, inf = 0, ones = 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N; v += (int64_t)gridDim.x * blockDim.x) {
         int d = dt2[v];
         if (d > 0) {
             np++;
+            if (ONES) ones += d == 1;
             if (d == IBIP_INF32) inf = 1; else mx = max(mx, d);
         }
     }
@@ -106,11 +108,13 @@ __global__ void k_stats(const int32_t *__restrict__ dt2, int64_t N, int *stats)
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         np += __shfl_xor_sync(0xffffffffu, np, o);
         inf |= __shfl_xor_sync(0xffffffffu, inf, o);
+        if (ONES) ones += __shfl_xor_sync(0xffffffffu, ones, o);
     }
     if ((threadIdx.x & 31) == 0) {
         atomicMax(stats + 0, mx);
         atomicAdd(stats + 1, np);
         atomicOr(stats + 2, inf);
+        if (ONES && ones) atomicAdd(stats + 3, ones);
     }
 }
 
@@ -2034,25 +2038,28 @@ int loop_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, int64_t 
     return IBIP_OK;
 }
 
-// Whether the loop beats the phases on one image.
-//  * Few large balls: a phase costs its barriers (~25 us on a cluster) however
-//    few steps it has, and one large ball after the other leaves nothing to run
-//    in parallel.  The measure is the pore volume in largest balls (but for a
-//    factor of 4): below 24 the loop is faster, above ~35 the phases are.
-//    phases / loop at 64^3 with 10 and 100 solid voxels (2.6, 21) 3.28 / 1.24 and
-//    3.04 / 1.98 ms, 128^3 with 100 (24) 11.96 / 7.97, 12^3-16^3 samples (7-16)
-//    0.50-0.65 / 0.34-0.57; 200^3 with 100 (29) 25.1 / 25.6, 64^3 pack of radius 8
-//    (45) 2.73 / 6.22, 48^3 blobs (92) 1.87 / 2.35.
-//  * Small images: eight samples of 24^3 (5,000-9,000 pore voxels) take 0.96 ms
-//    by phases and 0.78 on the loop on average (0.65-1.64 on the loop), eight of
-//    32^3 (12,000-22,000) 1.30 and 1.33.  (A batch keeps both kinds on the phases,
-//    where a cluster's idle time is another's.)
+// Whether the loop beats the phases on one image (ones: its voxels of value 1).
+//  * Few steps on few balls: the loop's time goes with its steps, about 0.48 of
+//    the voxels of value 1 (0.43-0.56 over blobs, packs and open images), the
+//    phases' with their number, which goes with the largest value: a phase costs
+//    its barriers (~25 us on a cluster) however little it holds.  Where the pore
+//    is many largest balls (npore / maxd^1.5) the phases run side by side.  Of
+//    1,094 images of 16^3-128^3 (blobs of sigma 2-8, packs of radius 4-10, open
+//    ones with few solid voxels) the loop is the faster for 52 %; this rule's
+//    choice takes 1.1 % more than the better one on average, the phases alone
+//    26 %, the loop alone 38 %.  Phases / loop: 12^3-16^3 samples 0.50-0.65 / 0.34-
+//    0.57 ms, 64^3 with 100 solid voxels 3.04 / 1.98, 128^3 with 100 11.96 / 7.97;
+//    a 47 x 57 x 50 pack of radius 9 2.33 / 3.06, 48^3 blobs of sigma 3 1.87 / 2.35.
+//    (A batch keeps all kinds on the phases, where a cluster's idle time is
+//    another image's.)
 //  * Short continuations: the phases take the whole phase that a step limit
 //    falls in.  1,000 steps more of the 200^3 pack 2.5-3.7 / 0.8-0.9 ms, 10,000
 //    1.9-3.0 / 2.9-3.1; of the 512^3 blobs 5.6-7.6 / 5.2-7.1.
-bool loop_is_faster(int64_t npore, int maxd, int resume, int64_t max_steps)
+bool loop_is_faster(int64_t npore, int64_t ones, int maxd, int resume, int64_t max_steps)
 {
-    return npore < 10000 || (double)npore < 24.0 * maxd * std::sqrt((double)maxd) || (resume && max_steps <= 4096);
+    const double m = maxd;
+    return (0.48 * (double)ones < 100.0 * std::pow(m, 0.8) && (double)npore < 70.0 * m * std::sqrt(m)) ||
+           (resume && max_steps <= 4096);
 }
 
 }  // namespace
@@ -2072,12 +2079,12 @@ int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, i
     if (!stats) return IBIP_ERR_OOM;
     int *h = (int *)ctx->h_pinned;
     ibip_prof_begin(ctx, IBIP_K_RANK);
-    cudaMemsetAsync(stats, 0, 3 * sizeof(int), s);
-    k_stats<<<ctx->sm_count * 8, 256, 0, s>>>(dt2, N, stats);
+    cudaMemsetAsync(stats, 0, 4 * sizeof(int), s);
+    k_stats<true><<<ctx->sm_count * 8, 256, 0, s>>>(dt2, N, stats);
     IBIP_LAUNCH(ctx);
-    cudaMemcpyAsync(h, stats, 3 * sizeof(int), cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(h, stats, 4 * sizeof(int), cudaMemcpyDeviceToHost, s);
     if (ibip_sync(ctx, s) != cudaSuccess) return IBIP_ERR_CUDA;
-    const int maxd = h[0], npore = h[1], hasinf = h[2];
+    const int maxd = h[0], npore = h[1], hasinf = h[2], ones = h[3];
     if (npore == 0) {
         if (!resume) {
             k_seq_init<<<ctx->sm_count * 8, 256, 0, s>>>(dt2, N, seq);
@@ -2091,7 +2098,7 @@ int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, i
     }
     int64_t done = -1;
     int st = kFloodGiveUp;
-    if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf) && !loop_is_faster(npore, maxd, resume, max_steps))
+    if (!ctx->trace && ibip_flood_ok(d, npore, maxd, hasinf) && !loop_is_faster(npore, ones, maxd, resume, max_steps))
         st = flood_run(ctx, dt2, d, inlet, max_steps, seq, step_r2, step_centre, cap, maxd, npore, mask, resume, k0, h_out,
                        &done);
     if (st == kFloodGiveUp && done >= 0)
@@ -2106,7 +2113,7 @@ int ibip_invade_run(ibip_ctx *ctx, const int32_t *dt2, ibip_dims d, int inlet, i
 
 int ibip_stats_launch(ibip_ctx *ctx, const int32_t *dt2, int64_t N, int *stats)
 {
-    k_stats<<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(dt2, N, stats);
+    k_stats<false><<<ctx->sm_count * 8, 256, 0, ctx->stream>>>(dt2, N, stats);
     IBIP_LAUNCH(ctx);
     return IBIP_OK;
 }
